@@ -111,6 +111,7 @@ struct axon_model {
   int* attn_cnt = nullptr;
   int max_splits = 1;
   int* err = nullptr;
+  AttnMaps attn_maps{};  // prefill attention
   CUtensorMap t_a{}, t_o{}, t_alo{};
   CUtensorMap t_a16{}, t_o16{}, t_alo16{};  // the same in boxes of 16 rows (decode GEMMs)
   CUtensorMap t_a64{}, t_o64{}, t_alo64{};  // and of 64 rows
@@ -692,6 +693,21 @@ struct VarlenBatch {
   int max_chunk;
 };
 
+// Whether a prefill's attention runs on the tcgen05 kernel (k_attn_tc.cu) or
+// on the mma.sync one. A tcgen05 CTA takes about 2 us longer to its first
+// output and holds a whole SM, so that the next kernels' CTAs cannot start
+// early beside it; it wins where key steps or waves amortise that. Whole
+// passes, mma.sync / tcgen05: 8B width 2 layers S = 256 418 / 424 us, 384 479 /
+// 477, 512 521 / 509; B = 16 S = 128 1365 / 1355, S = 256 2644 / 2606; 0.5B
+// width 4 layers S = 384 366 / 370, 512 380 / 378, B = 16 S = 256 853 / 841.
+// Variable-length batches may hold long contexts behind short chunks (8B width,
+// 30 contexts of up to 600 tokens and a 64-token chunk: 451 / 438) and take it
+// unless they have GEMV-sized projections (at most 64 rows).
+bool attn_on_tcgen05(int M, int S, bool varlen) {
+  if (varlen) return M > 64;
+  return S > 384 || (S >= 256 && M >= 2048);
+}
+
 int enqueue_prefill(axon_model* m, const int32_t* ids, int B, int S, const int32_t* bt, int logits_mode, float* logits,
                     int32_t* next, cudaStream_t st, Prof* pf = nullptr, const VarlenBatch* vl = nullptr) {
   const int M = vl ? vl->T : B * S;
@@ -704,6 +720,7 @@ int enqueue_prefill(axon_model* m, const int32_t* ids, int B, int S, const int32
                whd = static_cast<double>(m->V) * m->D * es;
   Proj pj{m, lc};
   const int D = m->D, Hd = m->H * m->d;
+  const bool attn_tc = !m->fp32 && attn_on_tcgen05(M, S, vl != nullptr);
   pbeg(pf, "embed");
   CK(launch_embed(lc, m->fp32, m->embed, m->V, D, ids, M, m->x, m->a, m->L > 0 ? m->layers[0].g1 : m->gf, m->ss,
                   m->Pmax, m->rinv, m->cfg.rms_norm_eps, m->err, m->a_lo));
@@ -734,7 +751,10 @@ int enqueue_prefill(axon_model* m, const int32_t* ids, int B, int S, const int32
     at.S = vl ? vl->max_chunk : S;
     const AttnVarlen avl{vl ? vl->cu : nullptr, vl ? vl->ctx : nullptr, M, rowmap};
     pbeg(pf, "prefill_attention");
-    CK(launch_attn_prefill(lc, m->fp32, at, B, vl ? &avl : nullptr));
+    if (attn_tc)
+      CK(launch_attn_prefill_tc(lc, at, m->attn_maps, l, B, vl ? &avl : nullptr));
+    else
+      CK(launch_attn_prefill(lc, m->fp32, at, B, vl ? &avl : nullptr));
     pend(pf, static_cast<double>(M) * (m->H + 2 * m->G) * m->d * es + static_cast<double>(M) * Hd * es,
          4.0 * B * m->H * m->d * (static_cast<double>(S) * (S + 1) / 2));
 
@@ -1114,7 +1134,7 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
   int major = 0;
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, m->device);
   if (major < 10) return fail(AXON_ERR_UNSUPPORTED);
-  if (prepare_attn_kernels() != cudaSuccess || prepare_gemm_kernels() != cudaSuccess ||
+  if (prepare_attn_kernels() != cudaSuccess || prepare_attn_tc_kernels() != cudaSuccess || prepare_gemm_kernels() != cudaSuccess ||
       prepare_gemv_kernels() != cudaSuccess)
     return fail(AXON_ERR_CUDA);
 
@@ -1439,7 +1459,10 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
 
   // ---- TMA descriptors (bf16 tensor-core path)
   if (!f32) {
-    bool ok = make_tma_2d_16(&m->t_a, m->a, Mcap, D, 128, m->f16) && make_tma_2d_16(&m->t_o, m->o, Mcap, Hd, 128, m->f16);
+    bool ok = m->L == 0 || make_attn_maps(&m->attn_maps, m->q, Mcap, m->kpool, m->vpool,
+                                          static_cast<long long>(m->L) * m->num_blocks * m->G * 16, m->H, m->G, m->d,
+                                          m->f16);
+    ok = ok && make_tma_2d_16(&m->t_a, m->a, Mcap, D, 128, m->f16) && make_tma_2d_16(&m->t_o, m->o, Mcap, Hd, 128, m->f16);
     if (ok && m->moe)
       ok = make_tma_2d_16(&m->t_asorted, m->moe_a_sorted, m->R_cap, D, 128, m->f16) &&
            make_tma_2d_16(&m->t_usorted, m->moe_u_sorted, m->R_cap, m->Fe, 128, m->f16);

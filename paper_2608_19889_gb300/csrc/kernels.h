@@ -147,6 +147,20 @@ cudaError_t launch_attn_decode(const LaunchCtx& lc, bool fp32, const AttnArgs& a
 // vl: variable-length batch, or null (B sequences of a.S tokens from position 0)
 cudaError_t launch_attn_prefill(const LaunchCtx& lc, bool fp32, const AttnArgs& a, int B,
                                 const AttnVarlen* vl = nullptr);
+// ---- prefill attention on the tensor cores (k_attn_tc.cu), 16-bit modes
+// Positions per 128-row query tile: PW positions x H/G heads of a kv head.
+inline int attn_tile_positions(int H, int G) { return 128 / (H / G); }
+struct AttnMaps {
+  CUtensorMap q;  // [rows][H][d], box PW positions x H/G heads x 64 dims
+  CUtensorMap k;  // the whole pool, [L * num_blocks * G * 16][d], box one 16-token block x 64 dims
+  CUtensorMap v;
+  int pool_rows = 0;
+};
+bool make_attn_maps(AttnMaps* maps, const void* q, long long rows, const void* kpool, const void* vpool,
+                    long long pool_rows, int H, int G, int d, bool f16);
+cudaError_t launch_attn_prefill_tc(const LaunchCtx& lc, const AttnArgs& a, const AttnMaps& maps, int layer, int B,
+                                   const AttnVarlen* vl = nullptr);
+cudaError_t prepare_attn_tc_kernels();
 // Key splits of the decode attention (1 .. min(max_blocks, 64)): the count
 // with the smallest estimated makespan over num_sms SMs, or, with
 // target_ctas > 0, as many as keep B x G x splits within that many CTAs.
@@ -174,6 +188,9 @@ struct GemmMaps {
   const GemmMaps* n128 = nullptr;  // the same operands with 128-row weight boxes (128-wide tiles), or null
 };
 bool make_tma_2d_16(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, bool f16);
+// [d2][d1][d0] 16-bit tensor, box box2 x box1 x 64 elements, 128-byte swizzle.
+bool make_tma_3d_16(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint32_t box1,
+                    uint32_t box2, bool f16);
 // Row-major [rows][cols] 16-bit matrix, box box_cols x box_rows, no swizzle
 // (dense rows in shared memory); out-of-range elements read as zero.
 bool make_tma_2d_plain(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_cols,
