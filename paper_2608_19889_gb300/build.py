@@ -16,7 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libaxon_gb300.so")
-SOURCES = ["api.cu", "k_gemv.cu", "k_attn.cu", "k_attn_tc.cu", "k_gemm.cu", "k_simt.cu", "k_persist.cu",
+SOURCES = ["api.cu", "k_gemv.cu", "k_attn.cu", "k_attn_tc.cu", "k_gemm.cu", "k_skinny.cu", "k_simt.cu", "k_persist.cu",
            "k_varlen.cu", "k_moe.cu", "noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr", "-I" + INCLUDE]

@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -112,6 +113,9 @@ struct axon_model {
   int max_splits = 1;
   int* err = nullptr;
   AttnMaps attn_maps{};  // prefill attention
+  // activation operands of the few-token projections: a, o, u by MLP width, gathered last rows
+  ActMaps am_a{}, am_o{}, am_last{};
+  std::map<int, ActMaps> am_u;
   CUtensorMap t_a{}, t_o{}, t_alo{};
   CUtensorMap t_a16{}, t_o16{}, t_alo16{};  // the same in boxes of 16 rows (decode GEMMs)
   CUtensorMap t_a64{}, t_o64{}, t_alo64{};  // and of 64 rows
@@ -126,13 +130,10 @@ struct axon_model {
   CUtensorMap* pmaps = nullptr;  // [4L + 1] weight maps, box 256 x 16
   PersistGrid* pgrid = nullptr;
   int persist_ctas = 0;
-  int decode_gemv_max = 32;  // decode projections with more tokens take the tcgen05 GEMM (AXON_DECODE_GEMV_MAX)
-  bool qkv_split = true;     // decode QKV of 9-16 tokens on the split-K GEMM (AXON_QKV_SPLITK=0: the GEMV)
   int persist_split_blocks = 16;  // persistent step: key blocks per split-KV item (AXON_PERSIST_SPLIT_BLOCKS)
   // decode attention grid budget in CTAs (AXON_ATTN_TARGET_CTAS; 0: the
   // split count with the smallest estimated makespan)
   int attn_target_ctas = 0;
-  GemmSplitK gemm_sk{};      // split-K workspace of the decode-sized tensor-core GEMMs
   // mixture of experts: routing and sorted-row workspace for up to Mcap
   // tokens (R_cap sorted rows)
   bool moe = false;
@@ -484,12 +485,32 @@ inline void pend(Prof* p, double bytes, double flops) {
   }
 }
 
+// Rows from which a pass runs its projections on the tcgen05 kernels (fewer:
+// the streaming GEMV). One line per model: mixed in a pass the two families
+// cost each other more than either loses (the GEMV keeps its loads in flight in
+// L1, the tcgen05 kernels claim nearly all of an SM's memory for staging, and
+// every change of that split drains the SM). Whole passes, GEMV / tcgen05:
+//   8B width, 2 layers: 4 tokens (qk-norm) 220 / 212 us, 8 tokens 235 / 224, 12
+//     tokens (fp16) 319 / 248, prompt of 2 tokens 232 / 206, of 64 (fp16) 817 / 281;
+//   16B mixture of experts, 2 layers (O projection 2048 x 2048): 1 token 174 / 187,
+//     4 tokens 223 / 232, 16 tokens 346 / 349;
+//   0.5B width, 4 layers: 24 tokens 216 / 190, 48 tokens 244 / 224, prompt of 32
+//     tokens 202 / 202, of 64 239 / 255;
+//   135M width, 6 layers: 16 tokens 193 / 211, 40 tokens (fp16) 339 / 248, prompt
+//     of 64 tokens 265 / 292.
+int tc_min_rows(const axon_model* m, bool decode) {
+  constexpr long long BIG = 1 << 23;  // weights of the smaller attention projection
+  if (std::min(static_cast<long long>(m->Nqkv) * m->D, static_cast<long long>(m->D) * m->H * m->d) >= BIG) return 1;
+  const bool wide_mlp = 2LL * m->F * m->D >= BIG / 4;
+  return m->f16 || (wide_mlp && decode) ? 24 : 65;
+}
+
 // One projection: picks the kernel for the mode and row count.
 struct Proj {
   const axon_model* m;
   LaunchCtx lc;
   bool decode = false;  // o_lo / u_lo were written by this step's producers
-  int gemv_max = 64;    // rows up to which the register-streaming GEMV runs (else the tcgen05 GEMM)
+  bool tc = false;      // the pass runs on the tcgen05 kernels
   cudaError_t rc = cudaSuccess;
   // act: activation rows (row stride act_stride elements), M rows. Returns
   // the norm state a RESID producer leaves behind.
@@ -498,48 +519,48 @@ struct Proj {
     ep.M = M;
     ep.N = N;
     NormState ns;
-    // Decode (gemv_max < 64) above 8 tokens, measured choices:
-    //  * the tcgen05 GEMM where its 128-wide tiles cover every SM (gate/up,
-    //    LM head);
-    //  * the residual projections (O, down) on the split-K GEMM where the
-    //    parts stay cheap to sum: a long K (>= 8192) or at most 16 tokens;
-    //    QKV too at most 16 tokens (qkv_split);
-    //  * otherwise the GEMV up to gemv_max tokens, the plain GEMM above.
-    const bool dec = gemv_max < 64 && maps != nullptr && !m->fp32 && M > 8;
-    const bool wide = dec && static_cast<long long>((N + 127) / 128) * ((M + 127) / 128) >= m->num_sms;
-    const bool split_kind =
-        (kind == EPI_RESID && (K >= 8192 || M <= 16)) || (kind == EPI_QKV && m->qkv_split && M <= 16);
-    const bool resid_split =
-        dec && !wide && split_kind && gemm_split_k(lc, M, N, K) > 1 && m->gemm_sk.ws != nullptr;
-    const bool gemv = (M <= gemv_max && !wide && !resid_split) || (!m->fp32 && maps == nullptr);
-    if (gemv && kind == EPI_RESID) {
-      ep.rinv_out = m->rinv;
-      ep.ticket = m->ticket;
-      ns.rinv = true;
+    // fp16 mode: the second term of the operand, where its producer left one
+    const void* lo = nullptr;
+    if (m->f16) {
+      if (act == m->a) lo = m->a_lo;
+      else if (decode && act == m->o) lo = m->o_lo;
+      else if (decode && act == m->u) lo = m->u_lo;
     }
-    if (gemv) {
-      // fp16 mode: consumers of the normed operand `a` also read its
-      // second term a_lo
-      const void* lo = nullptr;
-      if (m->f16) {
-        if (act == m->a) lo = m->a_lo;
-        else if (decode && act == m->o) lo = m->o_lo;
-        else if (decode && act == m->u) lo = m->u_lo;
+    if (!tc && (M <= 64 || (!m->fp32 && maps == nullptr))) {
+      if (kind == EPI_RESID) {
+        ep.rinv_out = m->rinv;
+        ep.ticket = m->ticket;
+        ns.rinv = true;
       }
       rc = launch_gemv(lc, kind, m->fp32, W, N, K, act, act_stride, M, ep, m->splitk, lo);
       ns.parts = N / 16;
-    } else if (m->fp32) {
-      rc = launch_gemm_simt(lc, kind, static_cast<const float*>(act), act_stride, static_cast<const float*>(W), M, N,
-                            K, ep);
-      ns.parts = N / 16;
-    } else {
-      int tn = gemm_tile_n(lc, *maps, M, N);
-      GemmSplitK sk = m->gemm_sk;
-      sk.ks = resid_split ? gemm_split_k(lc, M, N, K) : 1;
-      if (sk.ks > 1) tn = 256;
-      rc = launch_gemm_tc(lc, kind, *maps, M, N, K, ep, tn, &sk);
-      ns.parts = (N + tn - 1) / tn;
+      return ns;
     }
+    if (m->fp32) {
+      rc = launch_gemm_simt(lc, kind, static_cast<const float*>(act), act_stride, static_cast<const float*>(W), M, N, K,
+                            ep);
+      ns.parts = N / 16;
+      return ns;
+    }
+    // up to 128 rows: weights as the wide operand, K split over a cluster,
+    // unless the tiles alone fill the GPU more than twice. Two terms up to 32
+    // rows (64 in a prefill), and always where the operand is split (QKV).
+    if (M <= 128 && act_stride == K) {
+      const ActMaps* am = nullptr;
+      if (act == m->a) am = &m->am_a;
+      if (act == m->o) am = &m->am_o;
+      if (act == m->u && m->am_u.count(K)) am = &m->am_u.find(K)->second;
+      const bool two = lo != nullptr && (maps->split || M <= (decode ? 32 : 64));
+      const SkinnyPlan pl = am ? skinny_plan(lc, M, N, K, two) : SkinnyPlan{};
+      if (pl.ks > 0) {
+        rc = launch_skinny(lc, kind, maps->n128->w, *am, M, N, K, ep, pl);
+        ns.parts = (N + 127) / 128;
+        return ns;
+      }
+    }
+    const int tn = gemm_tile_n(lc, *maps, M, N);
+    rc = launch_gemm_tc(lc, kind, *maps, M, N, K, ep, tn);
+    ns.parts = (N + tn - 1) / tn;
     return ns;
   }
 };
@@ -629,7 +650,7 @@ int enqueue_mlp(axon_model* m, int l, Proj& pj, const LaunchCtx& lc, Prof* pf, c
     g.rinv = m->moe_ones;  // the sorted rows are normalised already
     g.rinv_stride = 0;
     pbeg(pf, decode ? "decode_moe_gateup" : "prefill_moe_gateup");
-    CK(launch_gemm_tc(lc, EPI_SWIGLU, w.m_gu_e, R, 2 * Fe, D, g, tn, nullptr, &grp));
+    CK(launch_gemm_tc(lc, EPI_SWIGLU, w.m_gu_e, R, 2 * Fe, D, g, tn, &grp));
     pend(pf, act * 2.0 * Fe * D * es + M * k * (D + Fe) * es, 2.0 * M * k * 2 * Fe * D);
     EpiArgs dn = base_epi(m);
     dn.M = R;
@@ -637,7 +658,7 @@ int enqueue_mlp(axon_model* m, int l, Proj& pj, const LaunchCtx& lc, Prof* pf, c
     dn.y_out = m->moe_y_sorted;
     dn.row_w = m->moe_row_w;
     pbeg(pf, decode ? "decode_moe_down" : "prefill_moe_down");
-    CK(launch_gemm_tc(lc, EPI_ROWSCALE, w.m_d_e, R, D, Fe, dn, tn, nullptr, &grp));
+    CK(launch_gemm_tc(lc, EPI_ROWSCALE, w.m_d_e, R, D, Fe, dn, tn, &grp));
     pend(pf, act * static_cast<double>(D) * Fe * es + M * k * (Fe * es + D * 4.0), 2.0 * M * k * D * Fe);
     EpiArgs cb = base_epi(m);
     cb.M = M;
@@ -711,6 +732,7 @@ bool attn_on_tcgen05(int M, int S, bool varlen) {
 int enqueue_prefill(axon_model* m, const int32_t* ids, int B, int S, const int32_t* bt, int logits_mode, float* logits,
                     int32_t* next, cudaStream_t st, Prof* pf = nullptr, const VarlenBatch* vl = nullptr) {
   const int M = vl ? vl->T : B * S;
+  const bool tc = !m->fp32 && (M > 64 || M >= tc_min_rows(m, false));
   LaunchCtx lc{st, m->use_pdl && !pf, m->num_sms, m->f16};
   const int2* rowmap = vl ? m->rowmap : nullptr;
   if (vl) CK(launch_varlen_rows(lc, vl->cu, vl->ctx, B, M, vl->max_chunk, m->cfg.max_context, m->rowmap, m->err));
@@ -719,6 +741,7 @@ int enqueue_prefill(axon_model* m, const int32_t* ids, int B, int S, const int32
   const double wq = static_cast<double>(m->Nqkv) * m->D * es, wo = static_cast<double>(m->D) * m->H * m->d * es,
                whd = static_cast<double>(m->V) * m->D * es;
   Proj pj{m, lc};
+  pj.tc = tc;
   const int D = m->D, Hd = m->H * m->d;
   const bool attn_tc = !m->fp32 && attn_on_tcgen05(M, S, vl != nullptr);
   pbeg(pf, "embed");
@@ -806,6 +829,11 @@ int enqueue_prefill(axon_model* m, const int32_t* ids, int B, int S, const int32
       hg.keys = m->keys + b0;
       hg.logits = logits ? logits + static_cast<size_t>(b0) * m->V : nullptr;
       const size_t off = static_cast<size_t>(b0) * D * m->esz;
+      const SkinnyPlan pl = tc ? skinny_plan(lc, nb, m->V, D, m->f16) : SkinnyPlan{};
+      if (pl.ks > 0) {
+        CK(launch_skinny(lc, EPI_LOGITS, m->v_head, m->am_last, nb, m->V, D, hg, pl, b0));
+        continue;
+      }
       CK(launch_gemv(lc, EPI_LOGITS, m->fp32, m->head, m->V, D, static_cast<char*>(m->a_last) + off, D, nb, hg,
                      m->splitk, m->a_lo_last ? static_cast<char*>(m->a_lo_last) + off : nullptr));
     }
@@ -901,14 +929,12 @@ PersistArgs persist_args(const axon_model* m, const int32_t* tokens, int B, int3
 int enqueue_decode(axon_model* m, const int32_t* tokens, int B, int32_t* ctx, const int32_t* bt, float* logits,
                    int32_t* next, cudaStream_t st, Prof* pf = nullptr, double kv_tokens = 0,
                    float* attn_part = nullptr, int* attn_cnt = nullptr, int attn_rows_cap = 0) {
-  LaunchCtx lc{st, m->use_pdl && !pf, m->num_sms, m->f16};
+  const bool tc = !m->fp32 && B >= tc_min_rows(m, true);
+  LaunchCtx lc{st, m->use_pdl && !pf, m->num_sms, m->f16, tc ? 100 : -1};
   g_trace_stream = st;
   Proj pj{m, lc};
   pj.decode = true;
-  // Above 32 tokens the GEMV's per-CTA re-reads of every activation row from
-  // L2 cost more than the weights; the tensor-core GEMM takes the 33..64
-  // tokens as one M tile and streams each weight tile once through TMA.
-  pj.gemv_max = m->decode_gemv_max;
+  pj.tc = tc;
   const int D = m->D, Hd = m->H * m->d;
   const double es = static_cast<double>(m->esz);
   const double wq = static_cast<double>(m->Nqkv) * m->D * es, wo = static_cast<double>(m->D) * Hd * es,
@@ -1112,11 +1138,6 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
     const int t = atoi(v);
     if (t >= 8 && t <= 4096) m->persist_split_blocks = t;
   }
-  if (const char* v = getenv("AXON_DECODE_GEMV_MAX")) {
-    const int t = atoi(v);
-    if (t >= 0 && t <= 64) m->decode_gemv_max = t;
-  }
-  if (const char* v = getenv("AXON_QKV_SPLITK")) m->qkv_split = atoi(v) != 0;
   g_trace = env_flag("AXON_TRACE");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   auto fail = [&](int code) {
@@ -1134,7 +1155,8 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
   int major = 0;
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, m->device);
   if (major < 10) return fail(AXON_ERR_UNSUPPORTED);
-  if (prepare_attn_kernels() != cudaSuccess || prepare_attn_tc_kernels() != cudaSuccess || prepare_gemm_kernels() != cudaSuccess ||
+  if (prepare_attn_kernels() != cudaSuccess || prepare_attn_tc_kernels() != cudaSuccess ||
+      prepare_skinny_kernels() != cudaSuccess || prepare_gemm_kernels() != cudaSuccess ||
       prepare_gemv_kernels() != cudaSuccess)
     return fail(AXON_ERR_CUDA);
 
@@ -1429,17 +1451,6 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
   m->splitk.ticket = static_cast<int*>(p);
   if (cudaMemsetAsync(m->splitk.ticket, 0, static_cast<size_t>(m->splitk.max_tiles) * 4, st) != cudaSuccess)
     return fail(AXON_ERR_CUDA);
-  if (!f32) {
-    // decode-sized tensor-core GEMMs with too few tiles split K (<= 128 rows)
-    const int nmax = std::max(std::max(m->Nqkv, 2 * F), std::max(D, V));
-    m->gemm_sk.max_tiles = (nmax + 255) / 256;
-    if ((rc = dev_alloc(m, &p, static_cast<size_t>(GEMM_MAX_UNITS) * 128 * 256 * 4))) return fail(rc);
-    m->gemm_sk.ws = static_cast<float*>(p);
-    if ((rc = dev_alloc(m, &p, static_cast<size_t>(m->gemm_sk.max_tiles) * 4))) return fail(rc);
-    m->gemm_sk.tickets = static_cast<int*>(p);
-    if (cudaMemsetAsync(m->gemm_sk.tickets, 0, static_cast<size_t>(m->gemm_sk.max_tiles) * 4, st) != cudaSuccess)
-      return fail(AXON_ERR_CUDA);
-  }
   m->max_splits = 64;
   const int dec_b = cfg->max_batch < 64 ? cfg->max_batch : 64;
   if ((rc = dev_alloc(m, &p, static_cast<size_t>(dec_b) * m->G * m->max_splits * 16 * (m->d + 2) * 4))) return fail(rc);
@@ -1473,6 +1484,12 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
     if (ok && m->a_lo)
       ok = make_tma_2d_16(&m->t_alo16, m->a_lo, Mcap, D, 16, m->f16) &&
            make_tma_2d_16(&m->t_alo64, m->a_lo, Mcap, D, 64, m->f16);
+    ok = ok && make_act_maps(&m->am_a, m->a, m->a_lo, Mcap, Mcap, D, m->f16) &&
+         make_act_maps(&m->am_o, m->o, m->o_lo, Mcap, m->cfg.max_batch, Hd, m->f16) &&
+         make_act_maps(&m->am_last, m->a_last, m->a_lo_last, m->cfg.max_batch, m->cfg.max_batch, D, m->f16);
+    for (const LayerW& w : m->layers)
+      if (w.Fl && !m->am_u.count(w.Fl))
+        ok = ok && make_act_maps(&m->am_u[w.Fl], m->u, m->u_lo, Mcap, m->cfg.max_batch, w.Fl, m->f16);
     auto small_a = [&](GemmMaps& g, const CUtensorMap& a16, const CUtensorMap& a64) {
       g.a16 = a16;
       g.a64 = a64;

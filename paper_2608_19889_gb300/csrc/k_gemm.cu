@@ -40,9 +40,7 @@ constexpr int NUM_THREADS = 192;
 // stored). Without the padding rows a stage is smaller, so more of them --
 // more weight bytes in flight per SM -- fit (up to 12).
 //
-// RING: the ring's byte budget. The residual kind at BN 256 keeps 8 KB of
-// static shared memory for its row sums, so its ring gets 196 KB.
-template <bool SPLIT, int BN_, int AROWS = 128, int RING = 200 * 1024>
+template <bool SPLIT, int BN_, int AROWS = 128>
 struct GCfg {
   static constexpr int BN = BN_;
   static constexpr int B_BYTES = BN * BK * 2;
@@ -52,16 +50,12 @@ struct GCfg {
   static constexpr int A_TILE = AROWS * BK * 2;  // bytes of one A term in a stage
   static constexpr int STAGE_BYTES = A_TERMS * A_TILE + B_BYTES;
   static constexpr int MAX_STAGES = SMALL ? 12 : 6;
+  static constexpr int RING = 200 * 1024;
   static constexpr int STAGES = RING / STAGE_BYTES > MAX_STAGES ? MAX_STAGES : RING / STAGE_BYTES;
   static_assert(!SMALL || STAGE_BYTES - (A_TERMS - 1) * A_TILE >= A_BYTES, "the MMA's 128-row read stays in its stage");
   static constexpr int BAR_BYTES = 8 * (2 * STAGES + 4) + 16;
   static constexpr int SMEM = STAGES * STAGE_BYTES + BAR_BYTES + 1024;
 };
-
-template <int KIND, int BN>
-constexpr int ring_budget() { return KIND == EPI_RESID && BN == 256 ? 196 * 1024 : 200 * 1024; }
-template <int KIND, bool SPLIT, int BN, int AROWS>
-using GCfgK = GCfg<SPLIT, BN, AROWS, ring_budget<KIND, BN>()>;
 
 // Residual epilogue staging: each epilogue warp's 32 rows x 32 accumulator
 // columns, rows padded to 36 floats (float4 stores of 8 consecutive rows
@@ -83,9 +77,8 @@ AXON_DEV void tile_coords(int t, int num_m, int num_n, int& mb, int& nb) {
 template <int KIND, typename T16, bool SPLIT, int BN_, int AROWS>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                   const __grid_constant__ CUtensorMap tmAlo, int M, int N, int K, EpiArgs ep, int ks, float* ws,
-                   int* tickets, GemmGroup grp) {
-  using C = GCfgK<KIND, SPLIT, BN_, AROWS>;
+                   const __grid_constant__ CUtensorMap tmAlo, int M, int N, int K, EpiArgs ep, GemmGroup grp) {
+  using C = GCfg<SPLIT, BN_, AROWS>;
   constexpr bool SMALL = C::SMALL;
   constexpr int BN = C::BN;
   constexpr int B_BYTES = C::B_BYTES;
@@ -142,17 +135,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   const bool grouped = grp.mb_expert != nullptr;
   const int num_m = grouped ? __ldcg(grp.n_mblocks) : (M + BM - 1) / BM, num_n = (N + BN - 1) / BN;
   const int tiles = num_m * num_n, KB = K / BK;
-  // Work units: (tile, K split) pairs, the ks splits of a tile adjacent.
-  // ks > 1 only with one M tile (M <= BM): each unit leaves its partial tile
-  // in `ws` and the last of a tile's units to finish sums them.
-  const int units = tiles * ks;
-
   if (warp == 0) {
     if (lane == 0) {
       int it = 0;
       bool ok = true;
-      for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
-        const int t = u / ks, sp = u - t * ks;
+      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
         int mb, nb;
         tile_coords(t, num_m, num_n, mb, nb);
         if (grouped) {
@@ -160,8 +147,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           nb = t - mb * num_n;
         }
         const int wrow = grouped ? __ldcg(grp.mb_expert + mb) * N + nb * BN : nb * BN;
-        const int kb1 = (sp + 1) * KB / ks;
-        for (int kb = sp * KB / ks; kb < kb1; ++kb, ++it) {
+        for (int kb = 0; kb < KB; ++kb, ++it) {
           const int s = it % STAGES;
           const uint32_t ph = (it / STAGES) & 1;
           if (!mbar_wait(empty_bar(s), ph ^ 1, ep.err)) {
@@ -181,15 +167,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       constexpr uint32_t idesc = idesc_f32acc(BM, BN, MmaFmt<T16>::v);
       int it = 0, lt = 0;
       bool ok = true;
-      for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++lt) {
-        const int sp = u % ks;
-        const int kb0 = sp * KB / ks, kb1 = (sp + 1) * KB / ks;
+      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++lt) {
         const int buf = lt & 1;
         const uint32_t aph = (lt >> 1) & 1;
         if (!mbar_wait(acce_bar(buf), aph ^ 1, ep.err)) break;
         tc_fence_after();
         const uint32_t d = tmem + buf * BN;
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
+        for (int kb = 0; kb < KB; ++kb, ++it) {
           const int s = it % STAGES;
           const uint32_t ph = (it / STAGES) & 1;
           if (!mbar_wait(full_bar(s), ph, ep.err)) {
@@ -201,7 +185,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           const uint64_t bd = smem_desc_sw128(b_at(s));
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)  // +32 bytes along K inside the swizzle atom
-            tc_mma_f16(d, ad + 2 * k, bd + 2 * k, idesc, (kb != kb0 || k != 0) ? 1u : 0u);
+            tc_mma_f16(d, ad + 2 * k, bd + 2 * k, idesc, (kb != 0 || k != 0) ? 1u : 0u);
           if (SPLIT) {
             const uint64_t ald = smem_desc_sw128(alo_at(s));
 #pragma unroll
@@ -216,13 +200,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   } else {
     const int q4 = warp & 3;  // TMEM lane quarter this warp may read
     const int row = q4 * 32 + lane;
-    const int etid = threadIdx.x - 64;  // 0..127 over the 4 epilogue warps
-    __shared__ int s_last;
-    __shared__ float s_rinv[BM];
-    __shared__ float s_ssp[KIND == EPI_RESID ? BM : 1][KIND == EPI_RESID ? BN / 16 : 1];
     int lt = 0;
-    for (int u = blockIdx.x; u < units; u += gridDim.x, ++lt) {
-      const int t = u / ks;
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++lt) {
       int mb, nb;
       tile_coords(t, num_m, num_n, mb, nb);
       if (grouped) {
@@ -235,90 +214,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       __syncwarp();
       if (!got) break;
       tc_fence_after();
-      if (ks > 1) {
-        // 1. this unit's partial tile -> workspace (rows < M; mb == 0)
-        const uint32_t taddr = tmem + (static_cast<uint32_t>(q4 * 32) << 16) + buf * BN;
-        float* wp = ws + (static_cast<long long>(u) * BM + row) * BN;
-#pragma unroll 1
-        for (int c = 0; c < BN; c += 16) {
-          uint32_t v[16];
-          tmem_ld16(taddr + c, v);
-          tmem_wait_ld();
-          if (row < M) {
-#pragma unroll
-            for (int i = 0; i < 16; i += 4)
-              *reinterpret_cast<float4*>(wp + c + i) =
-                  make_float4(__uint_as_float(v[i]), __uint_as_float(v[i + 1]), __uint_as_float(v[i + 2]),
-                              __uint_as_float(v[i + 3]));
-          }
-        }
-        tc_fence_before();
-        mbar_arrive(acce_bar(buf));
-        // ticket after the epilogue warps' barrier: one acquire-release atomic
-        // publishes the four warps' partial stores and, for the last unit,
-        // orders its loads of the other units' partials after theirs
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (etid == 0) s_last = (atom_add_acq_rel_gpu(tickets + t, 1) == ks - 1);
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (s_last) {
-          // 2. last unit of the tile: sum the ks partials in split order
-          // (deterministic) and run the epilogue, as (row, 16 columns) tasks
-          if (KIND != EPI_RESID && etid < M) s_rinv[etid] = row_rinv(ep, etid);
-          asm volatile("bar.sync 1, 128;" ::: "memory");
-          constexpr int CH = BN / 16;
-          for (int task = etid; task < M * CH; task += 128) {
-            const int m = task / CH, c = (task - m * CH) * 16;
-            const int n0 = nb * BN + c;
-            if (n0 >= N) continue;
-            float f[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) f[i] = 0.f;
-            // four splits' loads in flight per round trip, added in split order
-            for (int sp0 = 0; sp0 < ks; sp0 += 4) {
-              float4 a4[4][4];
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                const bool in = sp0 + u < ks;
-                const float* pp = ws + ((static_cast<long long>(t) * ks + (in ? sp0 + u : 0)) * BM + m) * BN + c;
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                  a4[u][i] = in ? __ldcg(reinterpret_cast<const float4*>(pp + 4 * i)) : make_float4(0.f, 0.f, 0.f, 0.f);
-              }
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                if (sp0 + u >= ks) break;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                  f[4 * i] += a4[u][i].x;
-                  f[4 * i + 1] += a4[u][i].y;
-                  f[4 * i + 2] += a4[u][i].z;
-                  f[4 * i + 3] += a4[u][i].w;
-                }
-              }
-            }
-            if (KIND == EPI_QKV) {
-              epi_qkv16<T16>(ep, m, n0, f, s_rinv[m]);
-            } else if (KIND == EPI_RESID) {
-              s_ssp[m][c >> 4] = epi_resid16<T16>(ep, m, n0, f);
-            } else if (KIND == EPI_SWIGLU) {
-              epi_swiglu16<T16>(ep, m, n0, f, s_rinv[m]);
-            } else {
-              argmax_commit(ep.keys + m, epi_logits16(ep, m, n0, f, s_rinv[m]));
-            }
-          }
-          asm volatile("bar.sync 1, 128;" ::: "memory");
-          if (KIND == EPI_RESID && etid < M) {
-            // the row's norm partial for this 256-wide tile, chunks summed in order
-            // (as the unsplit tile would); chunks past N count zero
-            float ssum = 0.f;
-            for (int c = 0; c < BN / 16; ++c)
-              if (nb * BN + c * 16 < N) ssum += s_ssp[etid][c];
-            ep.ss_out[static_cast<long long>(etid) * ep.ss_out_stride + nb] = ssum;
-          }
-          if (etid == 0) tickets[t] = 0;
-        }
-        continue;
-      }
       const int m = mb * BM + row;
       const bool mval = m < M && (!grp.row_valid || grp.row_valid[m] >= 0);
       float rinv = 1.f;
@@ -459,14 +354,14 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 
 template <int KIND, typename T16, bool SPLIT, int BN, int AROWS>
 cudaError_t launch_kind(const LaunchCtx& lc, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
-                        const GemmSplitK& sk, const GemmGroup& grp) {
-  const int tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN) * sk.ks;
+                        const GemmGroup& grp) {
+  const int tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
   // grouped: the tile count is known only on the device; one CTA per SM
   const int grid = grp.mb_expert ? lc.num_sms : (tiles < lc.num_sms ? tiles : lc.num_sms);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(NUM_THREADS);
-  cfg.dynamicSmemBytes = GCfgK<KIND, SPLIT, BN, AROWS>::SMEM + epi_smem<KIND>();
+  cfg.dynamicSmemBytes = GCfg<SPLIT, BN, AROWS>::SMEM + epi_smem<KIND>();
   cfg.stream = lc.stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -476,8 +371,7 @@ cudaError_t launch_kind(const LaunchCtx& lc, const GemmMaps& maps, int M, int N,
   const GemmMaps& g = BN == 256 ? maps : *maps.n128;
   const CUtensorMap& ta = AROWS == 16 ? g.a16 : (AROWS == 64 ? g.a64 : g.a);
   const CUtensorMap& tlo = SPLIT ? (AROWS == 16 ? g.a_lo16 : (AROWS == 64 ? g.a_lo64 : g.a_lo)) : ta;
-  return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<KIND, T16, SPLIT, BN, AROWS>, ta, g.w, tlo, M, N, K, ep, sk.ks,
-                            sk.ws, sk.tickets, grp);
+  return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<KIND, T16, SPLIT, BN, AROWS>, ta, g.w, tlo, M, N, K, ep, grp);
 }
 
 }  // namespace
@@ -525,7 +419,7 @@ template <int KIND, typename T16, bool SPLIT, int BN, int AROWS>
 cudaError_t set_smem1() {
   return cudaFuncSetAttribute(gemm_tc_kernel<KIND, T16, SPLIT, BN, AROWS>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              GCfgK<KIND, SPLIT, BN, AROWS>::SMEM + epi_smem<KIND>());
+                              GCfg<SPLIT, BN, AROWS>::SMEM + epi_smem<KIND>());
 }
 template <int KIND, typename T16, bool SPLIT>
 cudaError_t set_smem() {
@@ -551,29 +445,29 @@ cudaError_t prepare_gemm_t() {
 }
 template <typename T16, int BN, int AROWS>
 cudaError_t launch_t(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
-                     const GemmSplitK& sk, const GemmGroup& grp) {
+                     const GemmGroup& grp) {
   switch (kind) {
     case EPI_QKV:
-      return maps.split ? launch_kind<EPI_QKV, T16, true, BN, AROWS>(lc, maps, M, N, K, ep, sk, grp)
-                        : launch_kind<EPI_QKV, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, sk, grp);
-    case EPI_RESID: return launch_kind<EPI_RESID, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, sk, grp);
-    case EPI_SWIGLU: return launch_kind<EPI_SWIGLU, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, sk, grp);
-    case EPI_ROWSCALE: return launch_kind<EPI_ROWSCALE, T16, false, BN, 128>(lc, maps, M, N, K, ep, sk, grp);
-    default: return launch_kind<EPI_LOGITS, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, sk, grp);
+      return maps.split ? launch_kind<EPI_QKV, T16, true, BN, AROWS>(lc, maps, M, N, K, ep, grp)
+                        : launch_kind<EPI_QKV, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, grp);
+    case EPI_RESID: return launch_kind<EPI_RESID, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, grp);
+    case EPI_SWIGLU: return launch_kind<EPI_SWIGLU, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, grp);
+    case EPI_ROWSCALE: return launch_kind<EPI_ROWSCALE, T16, false, BN, 128>(lc, maps, M, N, K, ep, grp);
+    default: return launch_kind<EPI_LOGITS, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, grp);
   }
 }
 template <int BN, int AROWS>
 cudaError_t launch_ar(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
-                      const GemmSplitK& sk, const GemmGroup& grp) {
-  return lc.f16 ? launch_t<f16, BN, AROWS>(lc, kind, maps, M, N, K, ep, sk, grp)
-                : launch_t<bf16, BN, AROWS>(lc, kind, maps, M, N, K, ep, sk, grp);
+                      const GemmGroup& grp) {
+  return lc.f16 ? launch_t<f16, BN, AROWS>(lc, kind, maps, M, N, K, ep, grp)
+                : launch_t<bf16, BN, AROWS>(lc, kind, maps, M, N, K, ep, grp);
 }
 template <int BN>
 cudaError_t launch_bn(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
-                      const GemmSplitK& sk, const GemmGroup& grp, int arows) {
-  if (arows == 16) return launch_ar<BN, 16>(lc, kind, maps, M, N, K, ep, sk, grp);
-  if (arows == 64) return launch_ar<BN, 64>(lc, kind, maps, M, N, K, ep, sk, grp);
-  return launch_ar<BN, 128>(lc, kind, maps, M, N, K, ep, sk, grp);
+                      const GemmGroup& grp, int arows) {
+  if (arows == 16) return launch_ar<BN, 16>(lc, kind, maps, M, N, K, ep, grp);
+  if (arows == 64) return launch_ar<BN, 64>(lc, kind, maps, M, N, K, ep, grp);
+  return launch_ar<BN, 128>(lc, kind, maps, M, N, K, ep, grp);
 }
 }  // namespace
 
@@ -596,39 +490,18 @@ cudaError_t prepare_gemm_kernels() {
 }
 
 cudaError_t launch_gemm_tc(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K,
-                           const EpiArgs& ep, int tile_n, const GemmSplitK* split, const GemmGroup* group) {
+                           const EpiArgs& ep, int tile_n, const GemmGroup* group) {
   if (M < 1 || N < 1 || K < BK || (K % BK)) return cudaErrorInvalidValue;
   const GemmGroup grp = group ? *group : GemmGroup{};
-  if (grp.mb_expert && (!grp.n_mblocks || (split && split->ks > 1) || (M % BM))) return cudaErrorInvalidValue;
+  if (grp.mb_expert && (!grp.n_mblocks || (M % BM))) return cudaErrorInvalidValue;
   if (kind == EPI_ROWSCALE && !grp.mb_expert) return cudaErrorInvalidValue;
-  GemmSplitK sk;
-  if (split && split->ks > 1) {
-    // one M tile, 256-wide tiles, at most GEMM_MAX_UNITS units, at least one K block per unit
-    const int tiles = (N + 255) / 256;
-    if (M > BM || tile_n != 256 || !split->ws || !split->tickets || tiles * split->ks > GEMM_MAX_UNITS ||
-        split->ks > K / BK || tiles > split->max_tiles)
-      return cudaErrorInvalidValue;
-    sk = *split;
-  }
   // at most 16 (64) rows -- one M block -- and activation boxes of 16 (64)
   // rows: the small-M stage layouts
   const bool dec = !grp.mb_expert && kind != EPI_ROWSCALE;
   const int arows = (dec && M <= 16 && maps.has16) ? 16 : ((dec && M <= 64 && maps.has64) ? 64 : 128);
   if (tile_n == 128) {
     if (!maps.n128) return cudaErrorInvalidValue;
-    return launch_bn<128>(lc, kind, maps, M, N, K, ep, sk, grp, arows);
+    return launch_bn<128>(lc, kind, maps, M, N, K, ep, grp, arows);
   }
-  return launch_bn<256>(lc, kind, maps, M, N, K, ep, sk, grp, arows);
-}
-
-int gemm_split_k(const LaunchCtx& lc, int M, int N, int K) {
-  if (M > BM) return 1;
-  const int tiles = (N + 255) / 256;
-  if (2 * tiles >= lc.num_sms) return 1;
-  int ks = lc.num_sms / tiles;
-  const int kmax = K / BK / 4;  // keep >= 4 K blocks per unit
-  if (ks > kmax) ks = kmax;
-  if (ks > 16) ks = 16;
-  if (tiles * ks > GEMM_MAX_UNITS) ks = GEMM_MAX_UNITS / tiles;
-  return ks < 2 ? 1 : ks;
+  return launch_bn<256>(lc, kind, maps, M, N, K, ep, grp, arows);
 }

@@ -14,7 +14,31 @@ struct LaunchCtx {
   bool pdl;
   int num_sms;
   bool f16 = false;  // 16-bit operands are fp16 (else bf16); ignored in fp32 mode
+  // Preferred shared-memory carveout in percent (-1: the driver's choice). A
+  // decode step on the tcgen05 kernels, which take half an SM's shared memory or
+  // more, asks for all of it in every kernel: changing the split drains the SM,
+  // and the next kernel's CTAs cannot start beside the running ones (32B width,
+  // 16 tokens, one layer: 245 -> 233 us). A prefill gains nothing (its LM head
+  // is a GEMV, which keeps its loads in flight in L1).
+  int carveout = -1;
 };
+
+// Launch attributes of a kernel of the chain: programmatic dependent launch
+// and the shared-memory carveout. Returns their count.
+inline int chain_attrs(const LaunchCtx& lc, cudaLaunchAttribute (&attr)[2]) {
+  int n = 0;
+  if (lc.pdl) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
+  if (lc.carveout >= 0) {
+    attr[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[n].val.sharedMemCarveout = static_cast<unsigned>(lc.carveout);
+    ++n;
+  }
+  return n;
+}
 
 // ---- decode projections (k_gemv.cu): out[b][n] = act[b] . W[n], B <= 64
 // tokens, 16 weight rows per CTA, fused epilogue `kind`. Projections with
@@ -195,18 +219,6 @@ bool make_tma_3d_16(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1
 // (dense rows in shared memory); out-of-range elements read as zero.
 bool make_tma_2d_plain(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_cols,
                        uint32_t box_rows, bool f16);
-// Split-K mode of the GEMM for M <= 128 rows (decode): the K blocks are cut
-// into ks parts; each (256-wide tile, part) unit leaves its fp32 partial
-// tile in ws ([unit][128][256], rows < M written) and the last unit of a
-// tile to finish (ticket per tile, zero between launches, reset by that
-// unit; nobody waits) sums the parts in order and runs the epilogue.
-constexpr int GEMM_MAX_UNITS = 320;
-struct GemmSplitK {
-  int ks = 1;
-  float* ws = nullptr;       // GEMM_MAX_UNITS * 128 * 256 floats
-  int* tickets = nullptr;    // [max_tiles]
-  int max_tiles = 0;
-};
 // Grouped mode (mixture of experts, stacked experts): the activation rows
 // are sorted by expert, each expert's rows padded to whole 128-row blocks;
 // m-block b belongs to expert mb_expert[b], and *n_mblocks blocks exist
@@ -222,11 +234,32 @@ struct GemmGroup {
 // tile_n: 256 or 128 (from gemm_tile_n); the residual epilogue writes one
 // norm partial per row and tile, i.e. ceil(N / tile_n) of them.
 cudaError_t launch_gemm_tc(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
-                           int tile_n = 256, const GemmSplitK* split = nullptr, const GemmGroup* group = nullptr);
+                           int tile_n = 256, const GemmGroup* group = nullptr);
 int gemm_tile_n(const LaunchCtx& lc, const GemmMaps& maps, int M, int N);
-// K split (1 = none) for a decode-sized M x N x K product whose 256-wide
-// tiles cannot fill half the GPU.
-int gemm_split_k(const LaunchCtx& lc, int M, int N, int K);
+
+// ---- projections of few tokens (k_skinny.cu): weights as the 128-row MMA
+// operand, K split over the CTAs of a cluster.
+constexpr int SKINNY_MAX_SMEM = 230400;  // of one CTA per SM; two share it
+// An activation operand (and its second 16-bit term) in boxes of 16, 32, 64 and 128 rows.
+struct ActMaps {
+  CUtensorMap t[4];
+  CUtensorMap l[4];
+  bool lo = false;
+};
+bool make_act_maps(ActMaps* maps, const void* act, const void* act_lo, long long rows, long long lo_rows, long long K,
+                   bool f16);
+struct SkinnyPlan {
+  int ks = 0;  // CTAs per tile (cluster size); 0: the kernel does not suit the product
+  int nt = 0;  // token columns of the MMA
+  int stages = 0;
+  bool lo = false;
+};
+SkinnyPlan skinny_plan(const LaunchCtx& lc, int M, int N, int K, bool lo);
+// w: weight map of 128-row boxes; the M tokens are rows row0 .. of act. The
+// residual kind writes one norm partial per row and 128 columns.
+cudaError_t launch_skinny(const LaunchCtx& lc, int kind, const CUtensorMap& w, const ActMaps& act, int M, int N, int K,
+                          const EpiArgs& ep, const SkinnyPlan& pl, int row0 = 0);
+cudaError_t prepare_skinny_kernels();
 
 // ---- fp32 debug projections (k_simt.cu): plain tiled CUDA-core GEMM with
 // the same epilogues, any M.
