@@ -125,10 +125,11 @@ struct axon_model {
   bool use_graphs = true;
   bool use_pdl = true;
   // persistent decode step (B <= PERSIST_MAX_B): device layer table, grid
-  // barrier state, CTAs per launch (0: not available)
+  // launch state and exchange buffers, CTAs per launch (0: not available)
   PersistLayer* players = nullptr;
   CUtensorMap* pmaps = nullptr;  // [4L + 1] weight maps, box 256 x 16
   PersistGrid* pgrid = nullptr;
+  uint4* persist_ll = nullptr;  // exchange buffers
   int persist_ctas = 0;
   int persist_split_blocks = 16;  // persistent step: key blocks per split-KV item (AXON_PERSIST_SPLIT_BLOCKS)
   // decode attention grid budget in CTAs (AXON_ATTN_TARGET_CTAS; 0: the
@@ -874,6 +875,17 @@ bool persist_eligible(const axon_model* m, int B) {
          persist_fits(m->d, m->f16, B, m->D, std::max(std::max(m->D, m->H * m->d), m->F));
 }
 
+// Exchange buffers of the persistent step (PersistArgs::ll_*, in their order),
+// in 16-byte vectors, for PERSIST_MAX_B tokens and the widest form: a vector per
+// operand value after a residual projection or gate/up (own lines per item), a word per value
+// elsewhere.
+constexpr int PERSIST_LL = 9;
+size_t persist_ll_vecs(const axon_model* m, int i) {
+  const size_t D = m->D, Hd = static_cast<size_t>(m->H) * m->d, Gd = static_cast<size_t>(m->G) * m->d, F = m->F;
+  const size_t vecs[PERSIST_LL] = {D, D, D / 2, D / 2, Hd / 2, Gd / 2, Gd / 2, Hd / 2, F / 2};
+  return vecs[i] * PERSIST_MAX_B;
+}
+
 PersistArgs persist_args(const axon_model* m, const int32_t* tokens, int B, int32_t* ctx, const int32_t* bt,
                          float* logits, int32_t* next, int splits, float* attn_part, int* attn_cnt) {
   PersistArgs a;
@@ -886,7 +898,6 @@ PersistArgs persist_args(const axon_model* m, const int32_t* tokens, int B, int3
   a.F = m->F;
   a.V = m->V;
   a.Nqkv = m->Nqkv;
-  a.Pmax = m->Pmax;
   a.B = B;
   a.max_pos = m->cfg.max_context;
   a.blocks_per_seq = m->blocks_per_seq;
@@ -903,16 +914,12 @@ PersistArgs persist_args(const axon_model* m, const int32_t* tokens, int B, int3
   a.head = m->head;
   a.gf = m->gf;
   a.rope = m->rope;
-  a.x = m->x;
-  a.a = m->a;
-  a.a_lo = m->a_lo;
-  a.ss = m->ss;
-  a.q = m->q;
-  a.q_lo = m->q_lo;
-  a.o = m->o;
-  a.u = m->u;
-  a.o_lo = m->o_lo;
-  a.u_lo = m->u_lo;
+  uint4** const ll[PERSIST_LL] = {&a.ll_ao, &a.ll_ad, &a.ll_xo, &a.ll_xd, &a.ll_q, &a.ll_k, &a.ll_v, &a.ll_o, &a.ll_u};
+  uint4* at = m->persist_ll;
+  for (int i = 0; i < PERSIST_LL; ++i) {
+    *ll[i] = at;
+    at += persist_ll_vecs(m, i);
+  }
   a.keys = m->keys;
   a.attn_part = attn_part;
   a.attn_cnt = attn_cnt;
@@ -1579,7 +1586,7 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
     m->m_head.n128 = &m->m_head128;
     if (!ok) return fail(AXON_ERR_CUDA);
   }
-  // ---- persistent decode step: layer table and grid barrier state
+  // ---- persistent decode step: layer table, exchange buffers and launch state
   // default for B <= PERSIST_MAX_B; AXON_NO_PERSIST=1 keeps the launch chain
   if (!f32 && !m->moe && !env_flag("AXON_NO_PERSIST") && (m->d == 64 || m->d == 128)) {
     const int per_sm = persist_ctas_per_sm(m->d, m->f16);
@@ -1622,6 +1629,11 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
       if ((rc = dev_alloc(m, &p, sizeof(PersistGrid)))) return fail(rc);
       m->pgrid = static_cast<PersistGrid*>(p);
       if (cudaMemsetAsync(m->pgrid, 0, sizeof(PersistGrid), st) != cudaSuccess) return fail(AXON_ERR_CUDA);
+      size_t vecs = 0;
+      for (int i = 0; i < PERSIST_LL; ++i) vecs += persist_ll_vecs(m, i);
+      if ((rc = dev_alloc(m, &p, vecs * sizeof(uint4)))) return fail(rc);
+      m->persist_ll = static_cast<uint4*>(p);
+      if (cudaMemsetAsync(m->persist_ll, 0, vecs * sizeof(uint4), st) != cudaSuccess) return fail(AXON_ERR_CUDA);
       m->persist_ctas = m->num_sms;  // one CTA per SM
     }
   }

@@ -23,9 +23,11 @@ AXON_DEV uint32_t swz(uint32_t base, int tok, int ch) {
 
 // Copy one (block, kv head) tile of 16 x HD bf16 into swizzled shared memory
 // with `nthreads` cooperating threads starting at `tid`.
-template <int HD>
+template <int HD, bool ROLLED = false>
 AXON_DEV void stage_tile(uint32_t dst, const uint16_t* src, bool valid, int tid, int nthreads) {
   constexpr int CH = HD / 8;
+  constexpr int UNROLL = ROLLED ? 1 : 8;
+#pragma unroll UNROLL
   for (int c = tid; c < 16 * CH; c += nthreads) {
     const int tok = c / CH, ch = c % CH;
     cp_async16_zfill(swz<HD>(dst, tok, ch), valid ? src + tok * HD + ch * 8 : src, valid);
@@ -276,6 +278,13 @@ AXON_DEV void dec_sync() {
     __syncthreads();
 }
 
+// The item's exchange with the rest of the step (LL): none, when q, the cache
+// and o are plain memory of earlier and later kernels; or flagged words, inside
+// the persistent step (k_persist.cu, LLAttn).
+struct NoLL {
+  static constexpr bool on = false;
+};
+
 // One decode work item: split s of the keys of (kv head g, sequence b), run
 // by DEC_WARPS warps (thread `tid` of them) with `sm` as staging memory
 // (decode_smem<HD>() bytes). Reads of q and of the merge partials bypass L1:
@@ -283,8 +292,8 @@ AXON_DEV void dec_sync() {
 // PAIR = 1: the caller guarantees a second term of q and at most 8 query
 // heads per kv head, so only the paired tile loop is compiled; PAIR = 0:
 // chosen at run time.
-template <int HD, typename T16, bool NAMED, int PAIR = 0, int STAGES = 2>
-AXON_DEV void attn_decode_item(const AttnArgs& p, int s, int g, int b, uint8_t* sm, int tid) {
+template <int HD, typename T16, bool NAMED, int PAIR = 0, int STAGES = 2, typename LL = NoLL>
+AXON_DEV void attn_decode_item(const AttnArgs& p, int s, int g, int b, uint8_t* sm, int tid, const LL& ll = LL()) {
   constexpr int TILE = 16 * HD * 2;
   const int warp = tid >> 5, lane = tid & 31, r = lane >> 2, q = lane & 3;
   const int HPG = p.H / p.G;
@@ -312,8 +321,8 @@ AXON_DEV void attn_decode_item(const AttnArgs& p, int s, int g, int b, uint8_t* 
     bool ok;
     const int blk = block_of(p, b, j, ok);
     const long long off = (static_cast<long long>(blk) * p.G + g) * 16 * HD;
-    stage_tile<HD>(wbase + stg * 2 * TILE, kp + off, ok, lane, 32);
-    stage_tile<HD>(wbase + stg * 2 * TILE + TILE, vp + off, ok, lane, 32);
+    stage_tile<HD, LL::on>(wbase + stg * 2 * TILE, kp + off, ok, lane, 32);
+    stage_tile<HD, LL::on>(wbase + stg * 2 * TILE + TILE, vp + off, ok, lane, 32);
     cp_async_commit();
   };
   // The first key/value tile is requested before q is read: the two round
@@ -326,14 +335,22 @@ AXON_DEV void attn_decode_item(const AttnArgs& p, int s, int g, int b, uint8_t* 
   const long long qoff = (static_cast<long long>(b) * p.H + g * HPG) * HD;
   const uint16_t* qg = static_cast<const uint16_t*>(p.q) + qoff;
   const bool paired = PAIR == 1 || (p.q_lo != nullptr && HPG <= 8);
-  const uint16_t* qg1 = paired ? static_cast<const uint16_t*>(p.q_lo) + qoff + r * HD : qg + (r + 8) * HD;
   uint32_t qa[HD / 16][4];
+  if constexpr (LL::on) {
+    ll.template load_q<HD>(qa, (static_cast<long long>(b) * p.H + g * HPG + r) * HD, r < HPG, q);
+  } else {
+  const uint16_t* qg1 = paired ? static_cast<const uint16_t*>(p.q_lo) + qoff + r * HD : qg + (r + 8) * HD;
   load_q<HD>(qa, r < HPG ? qg + r * HD : nullptr, (paired ? r : r + 8) < HPG ? qg1 : nullptr, q);
+  }
+  // LL: the newest token's key and value have not reached the cache; they
+  // replace their row of the staged block
+  const int jnew = LL::on && p.ctx[b] + 1 == T ? (T - 1) >> 4 : -1;
 
   WarpState<HD> st;
   st.init();
   auto run_tiles = [&](auto paired_tag) {
     constexpr bool PAIRED = decltype(paired_tag)::value;
+#pragma unroll 1
     for (; j < je; j += DEC_WARPS) {
       const int jn = j + DEC_WARPS;
       if (STAGES == 2 && jn < je) {
@@ -343,6 +360,12 @@ AXON_DEV void attn_decode_item(const AttnArgs& p, int s, int g, int b, uint8_t* 
         cp_async_wait<0>();
       }
       __syncwarp();
+      if constexpr (LL::on) {
+        if (j == jnew) {
+          ll.template patch<HD>(wbase + stg * 2 * TILE, (static_cast<long long>(b) * p.G + g) * HD, (T - 1) & 15, lane);
+          __syncwarp();
+        }
+      }
       attn_tile16<HD, T16, PAIRED>(wbase + stg * 2 * TILE, wbase + stg * 2 * TILE + TILE, qa, st, j * 16, klo, T - 1,
                                    klo, T - 1, p.scale_log2, lane);
       __syncwarp();
@@ -390,6 +413,7 @@ AXON_DEV void attn_decode_item(const AttnArgs& p, int s, int g, int b, uint8_t* 
 
   const int rowlen = HD + 2;
   float* part = p.part + ((static_cast<long long>(b) * p.G + g) * p.splits) * 16 * rowlen;
+#pragma unroll 1
   for (int idx = tid; idx < HPG * HD; idx += DEC_WARPS * 32) {
     const int i = idx / HD, dd = idx - i * HD;
     float M = NEG_INF;
@@ -407,6 +431,10 @@ AXON_DEV void attn_decode_item(const AttnArgs& p, int s, int g, int b, uint8_t* 
     if (n_used == 1) {
       T16* og = static_cast<T16*>(p.o) + (static_cast<long long>(b) * p.H + g * HPG + i) * HD + dd;
       const float ov = L > 0.f ? O / L : 0.f;
+      if constexpr (LL::on) {
+        ll.template store_o<T16>((static_cast<long long>(b) * p.H + g * HPG + i) * HD + dd, ov);
+        continue;
+      }
       *og = from_f<T16>(ov);
       if (p.o_lo) static_cast<T16*>(p.o_lo)[og - static_cast<T16*>(p.o)] = from_f<T16>(ov - to_f(from_f<T16>(ov)));
     } else {
@@ -426,20 +454,28 @@ AXON_DEV void attn_decode_item(const AttnArgs& p, int s, int g, int b, uint8_t* 
   // acquire (passed on by the second barrier) the other CTAs'.
   __shared__ int is_last;
   dec_sync<NAMED>();
-  if (tid == 0) is_last = (atom_add_acq_rel_gpu(p.counter + b * p.G + g, 1) == n_used - 1);
+  if (tid == 0) {
+    is_last = (atom_add_acq_rel_gpu(p.counter + b * p.G + g, 1) == n_used - 1);
+    // LL: re-armed before this item's results leave, since nothing else orders
+    // it before the next layer's arrivals
+    if (LL::on && is_last) is_last = atomicExch(p.counter + b * p.G + g, 0) != 0;
+  }
   dec_sync<NAMED>();
   if (!is_last) return;
   // Each thread folds the n_used (m, l, O) partial states of its outputs in
   // split order with the online-softmax update; the loads of sixteen splits
   // are issued together, so up to sixteen splits cost one L2 round trip.
+#pragma unroll 1
   for (int idx = tid; idx < HPG * HD; idx += DEC_WARPS * 32) {
     const int i = idx / HD, dd = idx - i * HD;
     const float* pc = part + static_cast<long long>(i) * rowlen;
     float M = NEG_INF, L = 0.f, O = 0.f;
-    for (int t0 = 0; t0 < n_used; t0 += 16) {
-      float mv[16], lv[16], ov[16];
+    constexpr int SB = LL::on ? 8 : 16;  // splits' loads in flight (the persistent step keeps its code small)
+#pragma unroll 1
+    for (int t0 = 0; t0 < n_used; t0 += SB) {
+      float mv[SB], lv[SB], ov[SB];
 #pragma unroll
-      for (int u = 0; u < 16; ++u) {
+      for (int u = 0; u < SB; ++u) {
         const bool in = t0 + u < n_used;
         const float* pr = pc + static_cast<long long>(in ? t0 + u : 0) * 16 * rowlen;
         mv[u] = in ? __ldcg(pr + HD) : NEG_INF;
@@ -447,7 +483,7 @@ AXON_DEV void attn_decode_item(const AttnArgs& p, int s, int g, int b, uint8_t* 
         ov[u] = in ? __ldcg(pr + dd) : 0.f;
       }
 #pragma unroll
-      for (int u = 0; u < 16; ++u) {
+      for (int u = 0; u < SB; ++u) {
         if (mv[u] == NEG_INF) continue;  // a split with no visible key
         const float nm = fmaxf(M, mv[u]);
         const float a = exp2f(M - nm), f = exp2f(mv[u] - nm);  // a = 0 while M = -inf
@@ -458,10 +494,14 @@ AXON_DEV void attn_decode_item(const AttnArgs& p, int s, int g, int b, uint8_t* 
     }
     T16* og = static_cast<T16*>(p.o) + (static_cast<long long>(b) * p.H + g * HPG + i) * HD + dd;
     const float res = L > 0.f ? O / L : 0.f;
+    if constexpr (LL::on) {
+      ll.template store_o<T16>((static_cast<long long>(b) * p.H + g * HPG + i) * HD + dd, res);
+      continue;
+    }
     *og = from_f<T16>(res);
     if (p.o_lo) static_cast<T16*>(p.o_lo)[og - static_cast<T16*>(p.o)] = from_f<T16>(res - to_f(from_f<T16>(res)));
   }
-  if (tid == 0) p.counter[b * p.G + g] = 0;
+  if (!LL::on && tid == 0) p.counter[b * p.G + g] = 0;
 }
 
 

@@ -282,15 +282,26 @@ struct PersistLayer {
   void* kc;            // this layer's K pool
   void* vc;            // this layer's V pool
 };
-// Grid barrier state: zero before a launch; the launch leaves it zero.
+// Launch state: zero before the first launch. exit counts the CTAs that are
+// done (the launch leaves it zero), epoch numbers the exchange flags.
 struct PersistGrid {
-  unsigned count;
+  unsigned epoch;
   unsigned exit;
   unsigned abort;
   unsigned pad;
 };
+// Constants of one kind of phase, the same in every layer (filled at launch).
+struct PersistPhase {
+  int K, items, rot_step;  // items of 16 rows; items mod CTAs
+  int KP;                  // operand columns staged at a time
+  int ss_off, vb_off;      // shared-memory offsets of the norm partials and the epilogue buffer
+  int cap;                 // items per epilogue batch
+  uint32_t inv_row, inv_row_last;  // x / (vectors per operand row) = x * inv >> 32, for whole pieces and the last
+  uint32_t inv_B;                  // x / B = x * inv_B >> 16, x < 32
+};
 struct PersistArgs {
-  int L, D, H, G, d, F, V, Nqkv, Pmax, B;
+  PersistPhase ph[5];  // QKV, O, gate/up, down, LM head
+  int L, D, H, G, d, F, V, Nqkv, B;
   int max_pos, blocks_per_seq, num_blocks, splits, window, act;
   float eps, inv_D, scale_log2;
   const PersistLayer* layers;  // device [L]
@@ -301,16 +312,18 @@ struct PersistArgs {
   const void* head;
   const float* gf;
   const float2* rope;
-  float* x;
-  void* a;
-  void* a_lo;  // fp16 mode: second term of a
-  float* ss;   // norm partials [B][Pmax]
-  void* q;
-  void* q_lo;  // second term of q (16-bit modes)
-  void* o;
-  void* u;
-  void* o_lo;  // fp16 mode: second terms of o and u
-  void* u_lo;
+  // Exchange buffers of flagged 8-byte words (k_persist.cu): operand with norm
+  // partials, and residual, after the O (..o) and the down projection (..d), q, the
+  // newest k and v, attention and SwiGLU outputs.
+  uint4* ll_ao;
+  uint4* ll_ad;
+  uint4* ll_xo;
+  uint4* ll_xd;
+  uint4* ll_q;
+  uint4* ll_k;
+  uint4* ll_v;
+  uint4* ll_o;
+  uint4* ll_u;
   unsigned long long* keys;
   float* attn_part;
   int* attn_cnt;
