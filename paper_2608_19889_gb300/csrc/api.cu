@@ -124,7 +124,7 @@ struct axon_model {
   std::map<GraphKey, cudaGraphExec_t> graphs;
   bool use_graphs = true;
   bool use_pdl = true;
-  // persistent decode step (B <= PERSIST_MAX_B): device layer table, grid
+  // persistent decode step (B <= PERSIST_MAX_B): device layer table,
   // launch state and exchange buffers, CTAs per launch (0: not available)
   PersistLayer* players = nullptr;
   CUtensorMap* pmaps = nullptr;  // [4L + 1] weight maps, box 256 x 16
@@ -561,7 +561,7 @@ struct Proj {
     }
     const int tn = gemm_tile_n(lc, *maps, M, N);
     rc = launch_gemm_tc(lc, kind, *maps, M, N, K, ep, tn);
-    ns.parts = (N + tn - 1) / tn;
+    ns.parts = 2 * ((N + tn - 1) / tn);
     return ns;
   }
 };

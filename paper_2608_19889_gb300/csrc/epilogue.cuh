@@ -158,37 +158,51 @@ struct QkvIn {
   float b[16];
 };
 
-AXON_DEV void load_qkv16(const EpiArgs& e, int m, int n0, QkvIn& in) {
+AXON_DEV void load_qkv16p(const EpiArgs& e, int pos, int n0, QkvIn& in) {
   const int Hd = e.H * e.d, Gd = e.G * e.d;
-  const int c = n0 < Hd ? n0 % e.d : (n0 < Hd + Gd ? (n0 - Hd) % e.d : (n0 - Hd - Gd) % e.d);
-  int b;
-  const int pos = row_seq_pos(e, m, b);
+  const int c = n0 & (e.d - 1);  // within its head (d is 64 or 128, every region a multiple of it)
   if (n0 < Hd + Gd) {
     const int pc = min(max(pos, 0), e.max_pos - 1);
     const float2* cs = e.rope + static_cast<long long>(pc) * (e.d >> 1) + (c >> 4) * 8;
+    // 64-byte aligned runs: two pairs, four biases per load
+    const float4* c4 = reinterpret_cast<const float4*>(cs);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) in.cs[i] = cs[i];
+    for (int i = 0; i < 4; ++i) {
+      const float4 t = c4[i];
+      in.cs[2 * i] = make_float2(t.x, t.y);
+      in.cs[2 * i + 1] = make_float2(t.z, t.w);
+    }
   }
 #pragma unroll
-  for (int i = 0; i < 16; ++i) in.b[i] = e.bias ? e.bias[n0 + i] : 0.f;
+  for (int i = 0; i < 4; ++i) {
+    const float4 t = e.bias ? reinterpret_cast<const float4*>(e.bias + n0)[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    in.b[4 * i] = t.x;
+    in.b[4 * i + 1] = t.y;
+    in.b[4 * i + 2] = t.z;
+    in.b[4 * i + 3] = t.w;
+  }
+}
+
+AXON_DEV void load_qkv16(const EpiArgs& e, int m, int n0, QkvIn& in) {
+  int b;
+  load_qkv16p(e, row_seq_pos(e, m, b), n0, in);
 }
 
 // q/k/v: scale by r, add bias, rotate q and k, store q to the q buffer and
 // k, v into the cache slot of (b, pos). `in`: the chunk's loaded inputs.
 template <typename T>
-AXON_DEV void epi_qkv16x(const EpiArgs& e, int m, int n0, const float* v, float r, const QkvIn& in) {
+AXON_DEV void epi_qkv16p(const EpiArgs& e, int m, int b, int pos, int n0, const float* v, float r, const QkvIn& in) {
   const int Hd = e.H * e.d, Gd = e.G * e.d;
   int region, head, c;
+  const int sh = e.d == 128 ? 7 : 6;  // heads of 128 or 64
   if (n0 < Hd) {
-    region = 0; head = n0 / e.d; c = n0 - head * e.d;
+    region = 0; head = n0 >> sh; c = n0 & (e.d - 1);
   } else if (n0 < Hd + Gd) {
-    region = 1; head = (n0 - Hd) / e.d; c = n0 - Hd - head * e.d;
+    region = 1; head = (n0 - Hd) >> sh; c = n0 & (e.d - 1);
   } else {
-    region = 2; head = (n0 - Hd - Gd) / e.d; c = n0 - Hd - Gd - head * e.d;
+    region = 2; head = (n0 - Hd - Gd) >> sh; c = n0 & (e.d - 1);
   }
   const int j0 = (c >> 4) * 8, half = e.d >> 1;
-  int b;
-  const int pos = row_seq_pos(e, m, b);
   float lo[8], hi[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
@@ -237,6 +251,13 @@ AXON_DEV void epi_qkv16x(const EpiArgs& e, int m, int n0, const float* v, float 
     store8<T>(dst, lo);
     store8<T>(dst + half, hi);
   }
+}
+
+template <typename T>
+AXON_DEV void epi_qkv16x(const EpiArgs& e, int m, int n0, const float* v, float r, const QkvIn& in) {
+  int b;
+  const int pos = row_seq_pos(e, m, b);
+  epi_qkv16p<T>(e, m, b, pos, n0, v, r, in);
 }
 
 template <typename T>

@@ -10,12 +10,18 @@
 //                 accumulators), one lane issues tcgen05.mma kind::f16
 //                 (M=128, N=256, K=16) and frees ring slots / publishes
 //                 finished accumulators with tcgen05.commit;
-//   warps 2..5  : epilogue -- each reads its 32 TMEM lanes (rows) 16 columns
-//                 at a time with tcgen05.ld and applies the fused epilogue,
-//                 overlapping the next tile's main loop (double-buffered
-//                 accumulators).
+//   warps 2..9  : epilogue -- two warps per 32 TMEM lanes (rows), half the
+//                 columns each, 32 at a time with tcgen05.ld, and the fused
+//                 epilogue, overlapping the next tile's main loop
+//                 (double-buffered accumulators).
 // Tiles are visited in groups of 8 M-blocks per N sweep so the A and W
 // working sets of the concurrently running CTAs stay L2-resident.
+// Eight epilogue warps: where a launch has one or two tiles per CTA the epilogue
+// is exposed, and four warps kept too few reads in flight (8B width, 1024 rows,
+// per CTA: O 19 -> 13 us, QKV 10 -> 3; 0.5B width, 512 rows: QKV 6.5-11 -> 2-4.5,
+// gate/up 9.5 -> 4.6). Measured and not kept: launching the next kernel and
+// requesting its first weights under the last epilogue (small widths 1-3% faster,
+// 8B width 2-6% slower).
 // Every mbarrier wait is bounded (DEVERR_TIMEOUT instead of a hang).
 #include "kernels.h"
 
@@ -25,7 +31,8 @@ namespace {
 
 constexpr int BM = 128, BK = 64, GROUP_M = 8;
 constexpr int A_BYTES = BM * BK * 2;  // 16 KB
-constexpr int NUM_THREADS = 192;
+constexpr int EPI_WARPS = 8;
+constexpr int NUM_THREADS = 64 + 32 * EPI_WARPS;
 
 // BN_: columns of the output tile (256, or 128 where 256-wide tiles leave
 // the last wave mostly empty). SPLIT: the A operand is the sum of two
@@ -40,7 +47,9 @@ constexpr int NUM_THREADS = 192;
 // stored). Without the padding rows a stage is smaller, so more of them --
 // more weight bytes in flight per SM -- fit (up to 12).
 //
-template <bool SPLIT, int BN_, int AROWS = 128>
+//
+// RING: the ring's byte budget (the residual kind's epilogue staging takes 32 KB).
+template <bool SPLIT, int BN_, int AROWS = 128, int RING = 200 * 1024>
 struct GCfg {
   static constexpr int BN = BN_;
   static constexpr int B_BYTES = BN * BK * 2;
@@ -50,19 +59,20 @@ struct GCfg {
   static constexpr int A_TILE = AROWS * BK * 2;  // bytes of one A term in a stage
   static constexpr int STAGE_BYTES = A_TERMS * A_TILE + B_BYTES;
   static constexpr int MAX_STAGES = SMALL ? 12 : 6;
-  static constexpr int RING = 200 * 1024;
   static constexpr int STAGES = RING / STAGE_BYTES > MAX_STAGES ? MAX_STAGES : RING / STAGE_BYTES;
   static_assert(!SMALL || STAGE_BYTES - (A_TERMS - 1) * A_TILE >= A_BYTES, "the MMA's 128-row read stays in its stage");
   static constexpr int BAR_BYTES = 8 * (2 * STAGES + 4) + 16;
   static constexpr int SMEM = STAGES * STAGE_BYTES + BAR_BYTES + 1024;
 };
 
+template <int KIND, bool SPLIT, int BN, int AROWS>
+using GCfgK = GCfg<SPLIT, BN, AROWS, (KIND == EPI_RESID ? 192 : 200) * 1024>;
+
 // Residual epilogue staging: each epilogue warp's 32 rows x 32 accumulator
-// columns, rows padded to 36 floats (float4 stores of 8 consecutive rows
-// hit distinct banks).
-constexpr int EPI_TP = 36;
+// columns; 16-byte chunk j of row r lies at chunk j ^ (r & 7), so that both the
+// row-wise stores and the 4-row loads hit distinct banks.
 template <int KIND>
-constexpr int epi_smem() { return KIND == EPI_RESID ? 4 * 32 * EPI_TP * 4 : 0; }
+constexpr int epi_smem() { return KIND == EPI_RESID ? EPI_WARPS * 32 * 32 * 4 : 0; }
 
 AXON_DEV void tile_coords(int t, int num_m, int num_n, int& mb, int& nb) {
   const int per_group = GROUP_M * num_n;
@@ -78,7 +88,7 @@ template <int KIND, typename T16, bool SPLIT, int BN_, int AROWS>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmAlo, int M, int N, int K, EpiArgs ep, GemmGroup grp) {
-  using C = GCfg<SPLIT, BN_, AROWS>;
+  using C = GCfgK<KIND, SPLIT, BN_, AROWS>;
   constexpr bool SMALL = C::SMALL;
   constexpr int BN = C::BN;
   constexpr int B_BYTES = C::B_BYTES;
@@ -112,7 +122,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(accf_bar(i), 1);
-      mbar_init(acce_bar(i), 128);
+      mbar_init(acce_bar(i), 32 * EPI_WARPS);
     }
     fence_mbar_init();
     fence_proxy_async();
@@ -135,6 +145,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   const bool grouped = grp.mb_expert != nullptr;
   const int num_m = grouped ? __ldcg(grp.n_mblocks) : (M + BM - 1) / BM, num_n = (N + BN - 1) / BN;
   const int tiles = num_m * num_n, KB = K / BK;
+
   if (warp == 0) {
     if (lane == 0) {
       int it = 0;
@@ -198,7 +209,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     }
     __syncwarp();
   } else {
-    const int q4 = warp & 3;  // TMEM lane quarter this warp may read
+    // two warps per TMEM lane quarter (the one that a warp may read), half the
+    // tile's columns each
+    const int q4 = warp & 3, half = (warp - 2) >> 2;
+    constexpr int HALF = BN / 2;
+    const int cb = half * HALF;
     const int row = q4 * 32 + lane;
     int lt = 0;
     for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++lt) {
@@ -210,14 +225,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       }
       const int buf = lt & 1;
       const uint32_t aph = (lt >> 1) & 1;
-      const bool got = mbar_wait(accf_bar(buf), aph, ep.err);
-      __syncwarp();
-      if (!got) break;
-      tc_fence_after();
       const int m = mb * BM + row;
       const bool mval = m < M && (!grp.row_valid || grp.row_valid[m] >= 0);
-      float rinv = 1.f;
+      float rinv = 1.f;  // read while the tile's products run
       if (KIND != EPI_RESID && KIND != EPI_ROWSCALE && mval) rinv = row_rinv(ep, m);
+      int seq = 0, pos = 0;
+      if (KIND == EPI_QKV && mval) pos = row_seq_pos(ep, m, seq);
+      const bool got = __all_sync(0xffffffffu, mbar_wait(accf_bar(buf), aph, ep.err));
+      if (!got) break;
+      tc_fence_after();
       unsigned long long best = 0ull;
       const uint32_t taddr = tmem + (static_cast<uint32_t>(q4 * 32) << 16) + buf * BN;
       if (KIND == EPI_RESID) {
@@ -225,7 +241,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         // rows x 32 accumulator columns, then every global access (residual
         // read, x, a and a_lo writes) covers 4 rows x 128 bytes per
         // instruction, lane (r, c) taking row 4i + r, columns 4c .. 4c+3.
-        float* tw = epi_tile + q4 * 32 * EPI_TP;
+        float* tw = epi_tile + (warp - 2) * 32 * 32;
         const int lr = lane >> 3, lc = (lane & 7) * 4;
         const int mrow = mb * BM + q4 * 32 + lr;  // + 4i: the lane's rows
         bool rv[8];
@@ -249,17 +265,17 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 #pragma unroll
         for (int i = 0; i < 8; ++i) rs[i] = 0.f;
         float4 xcur[8], xnext[8];
-        load_x(0, xcur);
+        load_x(cb, xcur);
 #pragma unroll 1
-        for (int c0 = 0; c0 < BN; c0 += 32) {
-          if (c0 + 32 < BN) load_x(c0 + 32, xnext);
+        for (int c0 = cb; c0 < cb + HALF; c0 += 32) {
+          if (c0 + 32 < cb + HALF) load_x(c0 + 32, xnext);
           uint32_t v[2][16];
           tmem_ld16(taddr + c0, v[0]);
           tmem_ld16(taddr + c0 + 16, v[1]);
           tmem_wait_ld();
 #pragma unroll
           for (int j = 0; j < 8; ++j)
-            *reinterpret_cast<float4*>(tw + lane * EPI_TP + 4 * j) =
+            *reinterpret_cast<float4*>(tw + lane * 32 + 4 * (j ^ (lane & 7))) =
                 make_float4(__uint_as_float(v[j >> 2][(j & 3) * 4]), __uint_as_float(v[j >> 2][(j & 3) * 4 + 1]),
                             __uint_as_float(v[j >> 2][(j & 3) * 4 + 2]), __uint_as_float(v[j >> 2][(j & 3) * 4 + 3]));
           __syncwarp();
@@ -270,7 +286,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             const int rl = 4 * i + lr;
             float part = 0.f;
             if (rv[i] && n < N) {
-              const float4 acc = *reinterpret_cast<const float4*>(tw + rl * EPI_TP + lc);
+              const float4 acc = *reinterpret_cast<const float4*>(tw + rl * 32 + (lc ^ (4 * (rl & 7))));
               const float4 xo = xcur[i];
               const float xn[4] = {xo.x + acc.x, xo.y + acc.y, xo.z + acc.z, xo.w + acc.w};
               const long long off = static_cast<long long>(mrow + 4 * i) * ep.N + n;
@@ -287,34 +303,48 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
               }
               part = ((xn[0] * xn[0] + xn[1] * xn[1]) + xn[2] * xn[2]) + xn[3] * xn[3];
             }
-            // the row's 32 columns: the 8 lanes of the row, fixed tree order
-            part += __shfl_xor_sync(0xffffffffu, part, 1);
-            part += __shfl_xor_sync(0xffffffffu, part, 2);
-            part += __shfl_xor_sync(0xffffffffu, part, 4);
             rs[i] += part;
           }
           __syncwarp();
 #pragma unroll
           for (int i = 0; i < 8; ++i) xcur[i] = xnext[i];
         }
+        // a row's half tile: the 8 lanes of the row, fixed tree order
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          rs[i] += __shfl_xor_sync(0xffffffffu, rs[i], 1);
+          rs[i] += __shfl_xor_sync(0xffffffffu, rs[i], 2);
+          rs[i] += __shfl_xor_sync(0xffffffffu, rs[i], 4);
+        }
         if ((lane & 7) == 0) {
 #pragma unroll
           for (int i = 0; i < 8; ++i)
-            if (rv[i]) ep.ss_out[static_cast<long long>(mrow + 4 * i) * ep.ss_out_stride + nb] = rs[i];
+            if (rv[i]) ep.ss_out[static_cast<long long>(mrow + 4 * i) * ep.ss_out_stride + 2 * nb + half] = rs[i];
         }
       }
 #pragma unroll 1
-      for (int c = 0; c < BN && KIND != EPI_RESID; c += 16) {
-        uint32_t v[16];
-        tmem_ld16(taddr + c, v);
+      for (int c2 = cb; c2 < cb + HALF && KIND != EPI_RESID; c2 += 32) {
+        uint32_t v2[2][16];
+        tmem_ld16(taddr + c2, v2[0]);
+        tmem_ld16(taddr + c2 + 16, v2[1]);
+        const int n2 = nb * BN + c2;
+        // both chunks' rotation pairs and biases are requested together
+        QkvIn in[KIND == EPI_QKV ? 2 : 1];
+        if (KIND == EPI_QKV && mval) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            if (n2 + 16 * h < N) load_qkv16p(ep, pos, n2 + 16 * h, in[KIND == EPI_QKV ? h : 0]);
+        }
         tmem_wait_ld();
-        const int n0 = nb * BN + c;
-        if (mval && n0 < N) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int n0 = n2 + 16 * h;
+          if (!mval || n0 >= N) continue;
           float f[16];
 #pragma unroll
-          for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v[i]);
+          for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v2[h][i]);
           if (KIND == EPI_QKV) {
-            epi_qkv16<T16>(ep, m, n0, f, rinv);
+            epi_qkv16p<T16>(ep, m, seq, pos, n0, f, rinv, in[KIND == EPI_QKV ? h : 0]);
           } else if (KIND == EPI_SWIGLU) {
             epi_swiglu16<T16>(ep, m, n0, f, rinv);
           } else if (KIND == EPI_ROWSCALE) {
@@ -361,7 +391,7 @@ cudaError_t launch_kind(const LaunchCtx& lc, const GemmMaps& maps, int M, int N,
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(NUM_THREADS);
-  cfg.dynamicSmemBytes = GCfg<SPLIT, BN, AROWS>::SMEM + epi_smem<KIND>();
+  cfg.dynamicSmemBytes = GCfgK<KIND, SPLIT, BN, AROWS>::SMEM + epi_smem<KIND>();
   cfg.stream = lc.stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -419,7 +449,7 @@ template <int KIND, typename T16, bool SPLIT, int BN, int AROWS>
 cudaError_t set_smem1() {
   return cudaFuncSetAttribute(gemm_tc_kernel<KIND, T16, SPLIT, BN, AROWS>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              GCfg<SPLIT, BN, AROWS>::SMEM + epi_smem<KIND>());
+                              GCfgK<KIND, SPLIT, BN, AROWS>::SMEM + epi_smem<KIND>());
 }
 template <int KIND, typename T16, bool SPLIT>
 cudaError_t set_smem() {

@@ -231,8 +231,8 @@ struct GemmGroup {
   const int* n_mblocks = nullptr;
   const int* row_valid = nullptr;
 };
-// tile_n: 256 or 128 (from gemm_tile_n); the residual epilogue writes one
-// norm partial per row and tile, i.e. ceil(N / tile_n) of them.
+// tile_n: 256 or 128 (from gemm_tile_n); the residual epilogue writes two
+// norm partials per row and tile, i.e. 2 * ceil(N / tile_n) of them.
 cudaError_t launch_gemm_tc(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
                            int tile_n = 256, const GemmGroup* group = nullptr);
 int gemm_tile_n(const LaunchCtx& lc, const GemmMaps& maps, int M, int N);
