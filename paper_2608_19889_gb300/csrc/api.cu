@@ -546,7 +546,11 @@ struct Proj {
     // up to 128 rows: weights as the wide operand, K split over a cluster,
     // unless the tiles alone fill the GPU more than twice. Two terms up to 32
     // rows (64 in a prefill), and always where the operand is split (QKV).
-    if (M <= 128 && act_stride == K) {
+    // Residual projections of more rows too while few tiles share a long K
+    // (whole passes, tcgen05 GEMM / this: 0.5B width, 4 layers, prompts of 129,
+    // 512, 1000 tokens 260 / 237, 314 / 293, 367 / 362 us; 8B width, 2 layers, 160
+    // tokens 376 / 353; at 96 tiles, 300 tokens, 438 / 512).
+    if (act_stride == K && (M <= 128 || kind == EPI_RESID)) {
       const ActMaps* am = nullptr;
       if (act == m->a) am = &m->am_a;
       if (act == m->o) am = &m->am_o;

@@ -1,6 +1,6 @@
 // Projections of few tokens (decode batches, short prompts) on tcgen05:
-// out[m][n] = act[m] . W[n] for M <= 128 tokens, fused epilogues as in
-// epilogue.cuh.
+// out[m][n] = act[m] . W[n] for M <= 128 tokens (more in tiles of 128, where a
+// product has few of them), fused epilogues as in epilogue.cuh.
 //
 // The product is bound by streaming W once. Here the weights are the 128-row
 // operand of the MMA and the tokens its N dimension (16, 32, 64 or 128), so that a
@@ -57,10 +57,10 @@ AXON_DEV float4 ld_cluster4(uint32_t addr, uint32_t rank) {
 // nt: token columns of the MMA (16, 32, 64, 128); lo: the activations are two
 // 16-bit terms (a second MMA set on the second one); stages of the ring.
 template <int KIND, typename T16>
-__global__ void __launch_bounds__(SK_THREADS)
+__global__ void __launch_bounds__(SK_THREADS, 2)
     skinny_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmA,
-                  const __grid_constant__ CUtensorMap tmAlo, int M, int N, int K, EpiArgs ep, int ks, int nt, int lo,
-                  int stages, int row0) {
+                  const __grid_constant__ CUtensorMap tmAlo, int M_all, int N, int K, EpiArgs ep, int ks, int nt, int lo,
+                  int stages, int row0, int tiles_m) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -98,7 +98,11 @@ __global__ void __launch_bounds__(SK_THREADS)
   const uint32_t tmem = *reinterpret_cast<const uint32_t*>(smem_raw + (tmem_slot - raw));
 
   const int rank = ks > 1 ? static_cast<int>(cluster_rank()) : 0;
-  const int tile = blockIdx.x / ks, n_tile = tile * SK_BN;
+  // tile: 128 weight rows x nt tokens; the token tiles of one weight tile are
+  // neighbours, so that its weights are read from memory once
+  const int tile = blockIdx.x / ks / tiles_m, n_tile = tile * SK_BN;
+  const int m_tile = (blockIdx.x / ks - tile * tiles_m) * nt;
+  const int M = min(M_all - m_tile, nt);  // tokens of this tile
   const int KB = K / 64, kb0 = rank * KB / ks, nkb = (rank + 1) * KB / ks - kb0;
 
   if (warp == 0) {
@@ -113,8 +117,8 @@ __global__ void __launch_bounds__(SK_THREADS)
       auto load_a = [&](int i) {
         const int s = i % stages;
         const uint32_t dst = base + s * stage_bytes + SK_W_BYTES;
-        tma_load_2d(dst, &tmA, full_bar(s), (kb0 + i) * 64, row0);
-        if (lo) tma_load_2d(dst + act_bytes, &tmAlo, full_bar(s), (kb0 + i) * 64, row0);
+        tma_load_2d(dst, &tmA, full_bar(s), (kb0 + i) * 64, row0 + m_tile);
+        if (lo) tma_load_2d(dst + act_bytes, &tmAlo, full_bar(s), (kb0 + i) * 64, row0 + m_tile);
       };
       const int ahead = nkb < stages ? nkb : stages;
       for (int i = 0; i < ahead; ++i) load_w(i);
@@ -160,9 +164,9 @@ __global__ void __launch_bounds__(SK_THREADS)
     for (int m = warp - 2; m < M; m += 6) {
       float r;
       if (ep.rinv) {
-        r = ep.rinv[static_cast<long long>(m) * ep.rinv_stride];
+        r = ep.rinv[static_cast<long long>(m_tile + m) * ep.rinv_stride];
       } else {
-        const float* p = ep.ss + static_cast<long long>(m) * ep.ss_stride;
+        const float* p = ep.ss + static_cast<long long>(m_tile + m) * ep.ss_stride;
         float s = 0.f;
         for (int i = lane; i < ep.ss_parts; i += 32) s += p[i];
         r = 1.0f / sqrtf(warp_sum(s) * ep.inv_D + ep.eps);
@@ -179,8 +183,8 @@ __global__ void __launch_bounds__(SK_THREADS)
   auto load_in = [&](int t) {
     const int m = rank + (t >> 3) * ks, n0 = n_tile + (t & 7) * 16;
     if (t >= mine * 8 || n0 >= N) return;
-    if (KIND == EPI_RESID) load_resid16(ep, m, n0, xin);
-    if (KIND == EPI_QKV) load_qkv16(ep, m, n0, qin);
+    if (KIND == EPI_RESID) load_resid16(ep, m_tile + m, n0, xin);
+    if (KIND == EPI_QKV) load_qkv16(ep, m_tile + m, n0, qin);
   };
   load_in(threadIdx.x);
 
@@ -236,27 +240,27 @@ __global__ void __launch_bounds__(SK_THREADS)
         }
       }
       if (KIND == EPI_QKV) {
-        epi_qkv16x<T16>(ep, m, n0, f, rinv_s[m], qin);
+        epi_qkv16x<T16>(ep, m_tile + m, n0, f, rinv_s[m], qin);
       } else if (KIND == EPI_RESID) {
-        ssum = epi_resid16x<T16>(ep, m, n0, f, xin);
+        ssum = epi_resid16x<T16>(ep, m_tile + m, n0, f, xin);
       } else if (KIND == EPI_SWIGLU) {
-        epi_swiglu16<T16>(ep, m, n0, f, rinv_s[m]);
+        epi_swiglu16<T16>(ep, m_tile + m, n0, f, rinv_s[m]);
       } else {
-        best = epi_logits16(ep, m, n0, f, rinv_s[m]);
+        best = epi_logits16(ep, m_tile + m, n0, f, rinv_s[m]);
       }
     }
     if (KIND == EPI_RESID) {
       // the row's norm partial of this tile, in a fixed order
 #pragma unroll
       for (int o = 1; o < 8; o <<= 1) ssum += __shfl_xor_sync(0xffffffffu, ssum, o);
-      if (on && c == 0) ep.ss_out[static_cast<long long>(m) * ep.ss_out_stride + tile] = ssum;
+      if (on && c == 0) ep.ss_out[static_cast<long long>(m_tile + m) * ep.ss_out_stride + tile] = ssum;
     } else if (KIND == EPI_LOGITS) {
 #pragma unroll
       for (int o = 1; o < 8; o <<= 1) {
         const unsigned long long k = __shfl_xor_sync(0xffffffffu, best, o);
         best = k > best ? k : best;
       }
-      if (on && c == 0) argmax_commit(ep.keys + m, best);
+      if (on && c == 0) argmax_commit(ep.keys + m_tile + m, best);
     }
   }
   __syncwarp();
@@ -267,7 +271,8 @@ template <int KIND, typename T16>
 cudaError_t launch_kind(const LaunchCtx& lc, const CUtensorMap& w, const CUtensorMap& a, const CUtensorMap& alo, int M,
                         int N, int K, const EpiArgs& ep, const SkinnyPlan& pl, int row0) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((N + SK_BN - 1) / SK_BN * pl.ks);
+  const int tiles_m = (M + pl.nt - 1) / pl.nt;
+  cfg.gridDim = dim3((N + SK_BN - 1) / SK_BN * tiles_m * pl.ks);
   cfg.blockDim = dim3(SK_THREADS);
   const int lo = pl.lo ? 1 : 0;
   cfg.dynamicSmemBytes = 1024 + pl.stages * (SK_W_BYTES + pl.nt * 128 * (1 + lo)) + SK_MISC;
@@ -287,7 +292,8 @@ cudaError_t launch_kind(const LaunchCtx& lc, const CUtensorMap& w, const CUtenso
   }
   cfg.attrs = attr;
   cfg.numAttrs = n;
-  return cudaLaunchKernelEx(&cfg, skinny_kernel<KIND, T16>, w, a, alo, M, N, K, ep, pl.ks, pl.nt, lo, pl.stages, row0);
+  return cudaLaunchKernelEx(&cfg, skinny_kernel<KIND, T16>, w, a, alo, M, N, K, ep, pl.ks, pl.nt, lo, pl.stages, row0,
+                            tiles_m);
 }
 
 template <typename T16>
@@ -354,14 +360,17 @@ bool make_act_maps(ActMaps* maps, const void* act, const void* act_lo, long long
 
 SkinnyPlan skinny_plan(const LaunchCtx& lc, int M, int N, int K, bool lo) {
   SkinnyPlan pl;
-  if (M < 1 || M > 128 || (K & 63)) return pl;
+  if (M < 1 || (K & 63)) return pl;
   pl.nt = M <= 16 ? 16 : (M <= 32 ? 32 : (M <= 64 ? 64 : 128));
   pl.lo = lo;
-  const int tiles = (N + SK_BN - 1) / SK_BN, KB = K / 64;
+  const int tiles_m = (M + pl.nt - 1) / pl.nt, tiles = (N + SK_BN - 1) / SK_BN * tiles_m, KB = K / 64;
   const int stage = SK_W_BYTES + pl.nt * 128 * (lo ? 2 : 1);
+  // More than 128 tokens: only where the tiles leave at least half the SMs without
+  // work and K is long enough to share.
+  if (tiles_m > 1 && (2 * tiles > lc.num_sms || K < 2048)) return pl;
   const int per_sm = pl.nt == 128 ? 1 : 2;
   if (tiles > per_sm * g_clusters[1]) return pl;
-  const int budget = (pl.nt == 128 ? SKINNY_MAX_SMEM : SKINNY_MAX_SMEM / 2) - 1024 - SK_MISC - 1024;
+  const int budget = (per_sm == 1 ? SKINNY_MAX_SMEM : SKINNY_MAX_SMEM / 2) - 1024 - SK_MISC - 1024;
   pl.stages = budget / stage;
   if (pl.stages > SK_MAX_STAGES) pl.stages = SK_MAX_STAGES;
   // As many CTAs per tile as the clusters resident at a time allow, with at
@@ -377,7 +386,7 @@ SkinnyPlan skinny_plan(const LaunchCtx& lc, int M, int N, int K, bool lo) {
 
 cudaError_t launch_skinny(const LaunchCtx& lc, int kind, const CUtensorMap& w, const ActMaps& act, int M, int N, int K,
                           const EpiArgs& ep, const SkinnyPlan& pl, int row0) {
-  if (pl.ks < 1 || pl.ks > 8 || M < 1 || M > pl.nt || N < 1 || (K & 63) || K / 64 < pl.ks || pl.stages < 2 ||
+  if (pl.ks < 1 || pl.ks > 8 || M < 1 || N < 1 || (K & 63) || K / 64 < pl.ks || pl.stages < 2 ||
       (pl.lo && !act.lo))
     return cudaErrorInvalidValue;
   const int i = pl.nt == 16 ? 0 : (pl.nt == 32 ? 1 : (pl.nt == 64 ? 2 : 3));

@@ -66,3 +66,20 @@ def test_decode_batches(B, prec, oracle, monkeypatch):
         assert ax.axon_check_device(m)[0] == 0
     finally:
         ax.axon_free(m)
+
+
+@pytest.mark.parametrize("prec", ["bf16", "fp16"])
+def test_more_rows_than_a_token_tile(prec, oracle):
+    """129-300 rows: the O projection (17 weight tiles, K = 4096) runs on two or
+    three token tiles, the last one ragged."""
+    ax = _ax()
+    w, o = oracle
+    m = create(WIDE, w, max_batch=2, max_context=160, max_prefill_tokens=300, fp16=prec == "fp16")
+    try:
+        for B, S in ((1, 129), (2, 128), (2, 150)):
+            ids = si.make_ids(B, S, WIDE["V"], seed=S)
+            lg, _ = run_prefill(m, ids, ax.AXON_LOGITS_ALL, WIDE["V"])
+            check(lg, o.prefill(ids, o.new_contiguous_cache(B, 160)), tol=TOL[prec], what=f"B={B} S={S} ({prec})")
+        assert ax.axon_check_device(m)[0] == 0
+    finally:
+        ax.axon_free(m)
