@@ -490,20 +490,23 @@ inline void pend(Prof* p, double bytes, double flops) {
 // the streaming GEMV). One line per model: mixed in a pass the two families
 // cost each other more than either loses (the GEMV keeps its loads in flight in
 // L1, the tcgen05 kernels claim nearly all of an SM's memory for staging, and
-// every change of that split drains the SM). Whole passes, GEMV / tcgen05:
-//   8B width, 2 layers: 4 tokens (qk-norm) 220 / 212 us, 8 tokens 235 / 224, 12
-//     tokens (fp16) 319 / 248, prompt of 2 tokens 232 / 206, of 64 (fp16) 817 / 281;
-//   16B mixture of experts, 2 layers (O projection 2048 x 2048): 1 token 174 / 187,
-//     4 tokens 223 / 232, 16 tokens 346 / 349;
-//   0.5B width, 4 layers: 24 tokens 216 / 190, 48 tokens 244 / 224, prompt of 32
-//     tokens 202 / 202, of 64 239 / 255;
-//   135M width, 6 layers: 16 tokens 193 / 211, 40 tokens (fp16) 339 / 248, prompt
-//     of 64 tokens 265 / 292.
-int tc_min_rows(const axon_model* m, bool decode) {
-  constexpr long long BIG = 1 << 23;  // weights of the smaller attention projection
-  if (std::min(static_cast<long long>(m->Nqkv) * m->D, static_cast<long long>(m->D) * m->H * m->d) >= BIG) return 1;
-  const bool wide_mlp = 2LL * m->F * m->D >= BIG / 4;
-  return m->f16 || (wide_mlp && decode) ? 24 : 65;
+// every change of that split drains the SM). Whole passes, GEMV / tcgen05, us:
+//   8B width, 2 layers: 4 tokens (qk-norm) 220 / 204, 8 tokens 234 / 210, prompt of
+//     2 tokens 232 / 199, of 64 (fp16) 817 / 245; 32B width, 1 layer, 2 tokens
+//     196 / 193, 8 tokens 206 / 195;
+//   16B mixture of experts, 2 layers (O projection 2048 x 2048): 1 token 169 / 174,
+//     8 tokens 253 / 252, 12 tokens 308 / 294, prompt of 4 tokens 204 / 210, of 9
+//     247 / 241, of 32 349 / 298;
+//   0.5B width, 4 layers: 9 tokens 178 / 164, 24 tokens 218 / 172, prompt of 9
+//     tokens 153 / 155, of 16 160 / 157, of 64 238 / 210;
+//   135M width, 6 layers: 9 tokens 180 / 189 (fp16 210 / 203), 16 tokens 192 / 193, 24
+//     tokens 232 / 198, prompt of 16 tokens 168 / 183, of 32 227 / 197.
+int tc_min_rows(const axon_model* m) {
+  const long long small =  // weights of the smaller attention projection
+      std::min(static_cast<long long>(m->Nqkv) * m->D, static_cast<long long>(m->D) * m->H * m->d);
+  if (small >= 1 << 23) return 1;
+  if (small >= 1 << 21) return 5;
+  return m->f16 || 2LL * m->F * m->D >= 1 << 21 ? 9 : 17;
 }
 
 // One projection: picks the kernel for the mode and row count.
@@ -737,7 +740,7 @@ bool attn_on_tcgen05(int M, int S, bool varlen) {
 int enqueue_prefill(axon_model* m, const int32_t* ids, int B, int S, const int32_t* bt, int logits_mode, float* logits,
                     int32_t* next, cudaStream_t st, Prof* pf = nullptr, const VarlenBatch* vl = nullptr) {
   const int M = vl ? vl->T : B * S;
-  const bool tc = !m->fp32 && (M > 64 || M >= tc_min_rows(m, false));
+  const bool tc = !m->fp32 && (M > 64 || M >= tc_min_rows(m));
   LaunchCtx lc{st, m->use_pdl && !pf, m->num_sms, m->f16};
   const int2* rowmap = vl ? m->rowmap : nullptr;
   if (vl) CK(launch_varlen_rows(lc, vl->cu, vl->ctx, B, M, vl->max_chunk, m->cfg.max_context, m->rowmap, m->err));
@@ -940,7 +943,7 @@ PersistArgs persist_args(const axon_model* m, const int32_t* tokens, int B, int3
 int enqueue_decode(axon_model* m, const int32_t* tokens, int B, int32_t* ctx, const int32_t* bt, float* logits,
                    int32_t* next, cudaStream_t st, Prof* pf = nullptr, double kv_tokens = 0,
                    float* attn_part = nullptr, int* attn_cnt = nullptr, int attn_rows_cap = 0) {
-  const bool tc = !m->fp32 && B >= tc_min_rows(m, true);
+  const bool tc = !m->fp32 && B >= tc_min_rows(m);
   LaunchCtx lc{st, m->use_pdl && !pf, m->num_sms, m->f16, tc ? 100 : -1};
   g_trace_stream = st;
   Proj pj{m, lc};

@@ -13,11 +13,11 @@
 // 64-row fp32 partials of a split through L2 cost more than the idle SMs).
 //
 // Measured against the kernels that it replaced (the GEMV up to 32 tokens, split-K
-// GEMM through L2, unsplit GEMM), per launch, cold: 8B width, 64 tokens in fp16,
-// QKV 36.9 -> 23.4 us, O 29.1 -> 16.4, gate/up 49.6 -> 44.6 (235 MB), down 52.8 ->
-// 31.0 (117 MB); 32B width, 16 tokens, QKV 25.1 -> 18.9, O 21.4 -> 17.3, down
-// 52.8 -> 53.2 (283 MB, 5.3 TB/s). About 7 us of each are fixed: launch, first
-// weights, cluster barrier, epilogue.
+// GEMM through L2, unsplit GEMM): 8B width, 64 tokens in fp16, one layer over a paged
+// cache 309 -> 229 us of which the attention takes 103 (QKV 36.9 -> 20 us, O 29 ->
+// 13, gate/up 50 -> 40 (235 MB), down 53 -> 29 (117 MB)); 32B width, 16 tokens, one
+// layer 253 -> 224 us. About 5 us of each launch are fixed: launch, first weights,
+// cluster barrier, epilogue.
 //
 //   warp 0 : TMA producer; requests the first stages' weights before the
 //            preceding kernel has finished (they depend on nothing);
@@ -33,7 +33,7 @@ constexpr int SK_BN = 128;                // weight rows per tile
 constexpr int SK_W_BYTES = SK_BN * 64 * 2;  // weights of a stage
 constexpr int SK_PITCH = SK_BN + 4;       // floats per token row of the partial tile
 constexpr int SK_MAX_STAGES = 12;
-constexpr int SK_MAX_KS = 8;
+constexpr int SK_MAX_KS = 5;
 constexpr int SK_MISC = 8 * (2 * SK_MAX_STAGES + 1) + 8 + 128 * 4;  // barriers, TMEM slot, norm scales
 
 AXON_DEV uint32_t cluster_rank() {
@@ -160,18 +160,28 @@ __global__ void __launch_bounds__(SK_THREADS, 2)
     __syncwarp();
   }
   grid_dep_wait();
+  // the tokens' norm scales, eight tokens' reads in flight per warp
   if (KIND != EPI_RESID && warp >= 2) {
-    for (int m = warp - 2; m < M; m += 6) {
-      float r;
-      if (ep.rinv) {
-        r = ep.rinv[static_cast<long long>(m_tile + m) * ep.rinv_stride];
-      } else {
-        const float* p = ep.ss + static_cast<long long>(m_tile + m) * ep.ss_stride;
-        float s = 0.f;
-        for (int i = lane; i < ep.ss_parts; i += 32) s += p[i];
-        r = 1.0f / sqrtf(warp_sum(s) * ep.inv_D + ep.eps);
+    if (ep.rinv) {
+      for (int m = threadIdx.x - 64; m < M; m += SK_THREADS - 64)
+        rinv_s[m] = ep.rinv[static_cast<long long>(m_tile + m) * ep.rinv_stride];
+    } else {
+      constexpr int U = 8;
+      for (int m0 = (warp - 2) * U; m0 < M; m0 += 6 * U) {
+        float s[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) s[u] = 0.f;
+        for (int i = lane; i < ep.ss_parts; i += 32) {
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (m0 + u < M) s[u] += ep.ss[static_cast<long long>(m_tile + m0 + u) * ep.ss_stride + i];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          s[u] = warp_sum(s[u]);
+          if (lane == 0 && m0 + u < M) rinv_s[m0 + u] = 1.0f / sqrtf(s[u] * ep.inv_D + ep.eps);
+        }
       }
-      if (lane == 0) rinv_s[m] = r;
     }
   }
 
@@ -216,6 +226,32 @@ __global__ void __launch_bounds__(SK_THREADS, 2)
     tmem_dealloc(tmem, cols);
   }
 
+  // ks > 1: the sums over the cluster, a token row (512 contiguous bytes of every
+  // peer) per warp and step, into this CTA's own rows behind the partials. (Read
+  // by the tasks themselves, 64 bytes per lane, the sums of 64 tokens took 7 us.)
+  const float* src = part;
+  if (ks > 1) {
+    float* const sums = part + nt * SK_PITCH;
+    src = sums;
+    for (int t = warp; t < mine; t += SK_THREADS / 32) {
+      const uint32_t at = base + ((rank + t * ks) * SK_PITCH + lane * 4) * 4;
+      float4 v[SK_MAX_KS];
+#pragma unroll
+      for (int r = 0; r < SK_MAX_KS; ++r)
+        if (r < ks) v[r] = ld_cluster4(at, r);
+      float4 s = v[0];
+#pragma unroll
+      for (int r = 1; r < SK_MAX_KS; ++r) {
+        if (r >= ks) break;
+        s.x += v[r].x;
+        s.y += v[r].y;
+        s.z += v[r].z;
+        s.w += v[r].w;
+      }
+      *reinterpret_cast<float4*>(sums + t * SK_PITCH + lane * 4) = s;
+    }
+    __syncthreads();
+  }
   for (int t0 = 0; t0 < mine * 8; t0 += SK_THREADS) {
     const int t = t0 + threadIdx.x;
     const int c = t & 7, m = rank + (t >> 3) * ks, n0 = n_tile + c * 16;
@@ -226,18 +262,12 @@ __global__ void __launch_bounds__(SK_THREADS, 2)
     if (on) {
       float f[16];
 #pragma unroll
-      for (int i = 0; i < 16; ++i) f[i] = 0.f;
-      const uint32_t src = base + (m * SK_PITCH + c * 16) * 4;
-      for (int r = 0; r < ks; ++r) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float4 v = ks > 1 ? ld_cluster4(src + 16 * i, r)
-                                  : *reinterpret_cast<const float4*>(part + m * SK_PITCH + c * 16 + 4 * i);
-          f[4 * i] += v.x;
-          f[4 * i + 1] += v.y;
-          f[4 * i + 2] += v.z;
-          f[4 * i + 3] += v.w;
-        }
+      for (int i = 0; i < 4; ++i) {
+        const float4 v = *reinterpret_cast<const float4*>(src + (t >> 3) * SK_PITCH + c * 16 + 4 * i);
+        f[4 * i] = v.x;
+        f[4 * i + 1] = v.y;
+        f[4 * i + 2] = v.z;
+        f[4 * i + 3] = v.w;
       }
       if (KIND == EPI_QKV) {
         epi_qkv16x<T16>(ep, m_tile + m, n0, f, rinv_s[m], qin);
@@ -326,7 +356,7 @@ cudaError_t prepare_t() {
 }  // namespace
 
 // Clusters of ks CTAs that fit the device at one CTA per SM (index ks).
-static int g_clusters[9] = {};
+static int g_clusters[SK_MAX_KS + 1] = {};
 
 cudaError_t prepare_skinny_kernels() {
   cudaError_t e = prepare_t<bf16>();
@@ -378,7 +408,7 @@ SkinnyPlan skinny_plan(const LaunchCtx& lc, int M, int N, int K, bool lo) {
   // activation rows every CTA of a tile reads again) a launch got no shorter,
   // and a second wave of clusters doubles it (8B width, 8 tokens, QKV, 3 / 4 / 5 /
   // 6 CTAs: 16.9 / 15.9 / 15.5 / 24.4 us; 64 tokens: 24.9 / 23.4 / 25.4 / 34.7).
-  int ks = pl.nt <= 32 ? 5 : 4;
+  int ks = pl.nt <= 32 ? SK_MAX_KS : 4;
   while (ks > 1 && (KB / ks < 4 || tiles > per_sm * g_clusters[ks])) --ks;
   pl.ks = ks;
   return pl;
@@ -386,7 +416,7 @@ SkinnyPlan skinny_plan(const LaunchCtx& lc, int M, int N, int K, bool lo) {
 
 cudaError_t launch_skinny(const LaunchCtx& lc, int kind, const CUtensorMap& w, const ActMaps& act, int M, int N, int K,
                           const EpiArgs& ep, const SkinnyPlan& pl, int row0) {
-  if (pl.ks < 1 || pl.ks > 8 || M < 1 || N < 1 || (K & 63) || K / 64 < pl.ks || pl.stages < 2 ||
+  if (pl.ks < 1 || pl.ks > SK_MAX_KS || M < 1 || N < 1 || (K & 63) || K / 64 < pl.ks || pl.stages < 2 ||
       (pl.lo && !act.lo))
     return cudaErrorInvalidValue;
   const int i = pl.nt == 16 ? 0 : (pl.nt == 32 ? 1 : (pl.nt == 64 ? 2 : 3));
