@@ -642,8 +642,7 @@ int enqueue_mlp(axon_model* m, int l, Proj& pj, const LaunchCtx& lc, Prof* pf, c
     EpiArgs nx = base_epi(m);
     set_norm(m, ns, nx);
     pbeg(pf, decode ? "decode_moe_route" : "prefill_moe_route");
-    CK(launch_moe_route_plan(lc, ma, M));
-    CK(launch_moe_gather(lc, ma, M, nx));
+    CK(launch_moe_route(lc, ma, M, nx));
     pend(pf, M * (E * 4.0 + D * (2 * es + es * k)), 0);
     // tile width: 128 when the experts' blocks alone leave most SMs idle
     const int tn = (static_cast<long long>(M) * k * ((D + 255) / 256) < m->num_sms) ? 128 : 256;

@@ -16,6 +16,7 @@
 //                       block count -- the grouped GEMM's tile list;
 //   moe_gather_kernel   the sorted operand rows: the normalised input
 //                       h = (a [+ a_lo]) * r, rounded once to 16 bits;
+//                       for few slots the plan kernel's CTA does this too;
 //   [grouped tcgen05 GEMM gate/up + SwiGLU, grouped GEMM down scaled by the
 //    row's weight: k_gemm.cu]
 //   moe_combine_kernel  per token: x += the sum of its k expert outputs in
@@ -30,6 +31,12 @@ constexpr int ROUTE_THREADS = 256;
 constexpr int PLAN_THREADS = 1024;
 // Token counts up to which one CTA both routes and sorts (the decode path).
 constexpr int FUSED_ROUTE_MAX_T = 256;
+// Slots up to which that CTA also gathers their rows: one per warp. Beyond
+// that the rows of one warp follow each other, while a launch of its own
+// spreads them over the chip (decode pass of 4 layers, 6 experts per token,
+// gathered here / by its own launch: 6 slots 338 / 343 us, 24 slots 491 / 493,
+// 42 slots 580 / 571, 96 slots 756 / 737).
+constexpr int FUSED_GATHER_MAX = 32;
 
 // Token t: softmax of its router logits, top-k by repeated arg-max over
 // (probability, lowest index), the weights (renormalised over the k chosen
@@ -103,100 +110,26 @@ __global__ void __launch_bounds__(ROUTE_THREADS) moe_route_kernel(MoeArgs a, int
   if (t < T) route_token(a, t, sh + warp * a.E, lane);
 }
 
-// Stable counting sort of the n = T * k slots by expert, in rounds of
-// PLAN_THREADS slots: within a warp, slots of one expert are ranked by
-// lane (match_any), warps are ranked in order by a per-expert prefix over
-// the round's warp counts, rounds in order by the running counts.
-// With ROUTE, the CTA's warps first route the T tokens themselves (the
-// per-warp scratch is the count table, unused until then).
-template <bool ROUTE>
-__global__ void __launch_bounds__(PLAN_THREADS) moe_plan_kernel(MoeArgs a, int T) {
-  grid_dep_launch();
-  grid_dep_wait();
-  __shared__ int cnt[MOE_MAX_EXPERTS];
-  __shared__ int seg[MOE_MAX_EXPERTS];
-  __shared__ int wcnt[PLAN_THREADS / 32][MOE_MAX_EXPERTS];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int E = a.E, n = T * a.k;
-  if (ROUTE) {
-    for (int t = warp; t < T; t += PLAN_THREADS / 32) route_token(a, t, reinterpret_cast<float*>(wcnt[warp]), lane);
-    __syncthreads();
-  }
-  for (int e = tid; e < E; e += PLAN_THREADS) cnt[e] = 0;
-  for (int base = 0; base < n; base += PLAN_THREADS) {
-    for (int c = tid; c < (PLAN_THREADS / 32) * E; c += PLAN_THREADS) wcnt[c / E][c % E] = 0;
-    __syncthreads();
-    const int i = base + tid;
-    int e = i < n ? a.topk_idx[i] : -1;
-    if (e >= E || e < -1) {
-      set_err(a.err, DEVERR_SEQ);
-      e = -1;
-    }
-    const unsigned peers = __match_any_sync(0xffffffffu, e);
-    const int rank_w = __popc(peers & ((1u << lane) - 1u));
-    if (e >= 0 && rank_w == 0) wcnt[warp][e] = __popc(peers);
-    __syncthreads();
-    for (int x = tid; x < E; x += PLAN_THREADS) {
-      int s = cnt[x];
-      for (int w = 0; w < PLAN_THREADS / 32; ++w) {
-        const int c = wcnt[w][x];
-        wcnt[w][x] = s;
-        s += c;
-      }
-      cnt[x] = s;
-    }
-    __syncthreads();
-    if (e >= 0) a.slot_row[i] = wcnt[warp][e] + rank_w;  // rank within the expert, for now
-    else if (i < n) a.slot_row[i] = -1;
-    __syncthreads();
-  }
-  if (tid == 0) {
-    int acc = 0;
-    for (int e = 0; e < E; ++e) {
-      seg[e] = acc;
-      const int blocks = (cnt[e] + 127) >> 7;
-      for (int b = 0; b < blocks; ++b) a.mb_expert[(acc >> 7) + b] = e;
-      acc += blocks << 7;
-    }
-    *a.n_mblocks = acc >> 7;
-  }
-  __syncthreads();
-  for (int i = tid; i < n; i += PLAN_THREADS) {
-    const int e = a.topk_idx[i];
-    const int rk = a.slot_row[i];
-    if (rk < 0 || e < 0 || e >= E) continue;
-    const int row = seg[e] + rk;
-    a.slot_row[i] = row;
-    a.row_tok[row] = i / a.k;
-    a.row_w[row] = a.topk_w[i];
-  }
-  // padding rows of each segment
-  for (int e = 0; e < E; ++e) {
-    const int pad0 = seg[e] + cnt[e], pad1 = seg[e] + (((cnt[e] + 127) >> 7) << 7);
-    for (int row = pad0 + tid; row < pad1; row += PLAN_THREADS) {
-      a.row_tok[row] = -1;
-      a.row_w[row] = 0.f;
-    }
-  }
-}
-
 // Sorted operand rows: slot i = (token t, j) goes to row slot_row[i] as the
 // normalised input h = (a [+ a_lo]) * r of token t, rounded once to 16 bits.
 // Padding rows are left as they are: a row of the grouped GEMMs' operand
 // only reaches its own output row, which the epilogues skip. One warp per
 // slot, 8 elements per lane step.
 template <typename T16>
-__global__ void __launch_bounds__(256) moe_gather_kernel(MoeArgs a, int T, EpiArgs ns) {
-  grid_dep_launch();
-  grid_dep_wait();
+AXON_DEV void gather_slots(const MoeArgs& a, int T, const EpiArgs& ns, int warp, int nwarps, int lane) {
   const int n = T * a.k, per_row = a.D / 8;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  const int nwarps = (gridDim.x * blockDim.x) >> 5;
   for (int i = warp; i < n; i += nwarps) {
     const int row = a.slot_row[i];
     if (row < 0) continue;
     const int t = i / a.k;
-    const float r = row_rinv(ns, t);
+    float r;
+    if (ns.rinv) {
+      r = ns.rinv[static_cast<long long>(t) * ns.rinv_stride];
+    } else {
+      float s = 0.f;
+      for (int j = lane; j < ns.ss_parts; j += 32) s += ns.ss[static_cast<long long>(t) * ns.ss_stride + j];
+      r = 1.0f / sqrtf(warp_sum(s) * ns.inv_D + ns.eps);
+    }
     const uint4* sh = reinterpret_cast<const uint4*>(static_cast<const T16*>(a.act) + t * a.act_stride);
     const uint4* sl = a.act_lo ? reinterpret_cast<const uint4*>(static_cast<const T16*>(a.act_lo) + t * a.act_stride)
                                : nullptr;
@@ -220,6 +153,119 @@ __global__ void __launch_bounds__(256) moe_gather_kernel(MoeArgs a, int T, EpiAr
       dh[c] = o;
     }
   }
+}
+
+// Stable counting sort of the n = T * k slots by expert, in rounds of
+// PLAN_THREADS slots: within a warp, slots of one expert are ranked by
+// lane (match_any), warps are ranked in order by a per-expert prefix over
+// the round's warp counts, rounds in order by the running counts.
+// With ROUTE, the CTA's warps first route the T tokens themselves (the
+// per-warp scratch is the count table, unused until then) and, for at most
+// FUSED_GATHER_MAX slots, also gather the sorted rows.
+//
+// One CTA, bound by the latency of its steps: only the warps that hold slots
+// are counted, the segments come from a warp scan over the experts, and each
+// warp pads the segments of its own experts. 64 experts of which 6 per token,
+// cold caches: 1 token, routed and gathered, 15.9 us and a gather launch of 7 ->
+// 14.1 us; 509 tokens 27 -> 12.2 us.
+template <bool ROUTE, typename T16>
+__global__ void __launch_bounds__(PLAN_THREADS) moe_plan_kernel(MoeArgs a, int T, EpiArgs ns, int gather) {
+  grid_dep_launch();
+  grid_dep_wait();
+  constexpr int WARPS = PLAN_THREADS / 32;
+  __shared__ int cnt[MOE_MAX_EXPERTS];
+  __shared__ int seg[MOE_MAX_EXPERTS];
+  __shared__ int wcnt[WARPS][MOE_MAX_EXPERTS];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int E = a.E, n = T * a.k;
+  if (ROUTE) {
+    for (int t = warp; t < T; t += WARPS) route_token(a, t, reinterpret_cast<float*>(wcnt[warp]), lane);
+    __syncthreads();
+  }
+  for (int e = tid; e < E; e += PLAN_THREADS) cnt[e] = 0;
+  for (int base = 0; base < n; base += PLAN_THREADS) {
+    const int used = min(WARPS, (n - base + 31) >> 5);  // warps with slots this round
+    for (int e = lane; e < E; e += 32) wcnt[warp][e] = 0;
+    __syncwarp();
+    const int i = base + tid;
+    int e = i < n ? a.topk_idx[i] : -1;
+    if (e >= E || e < -1) {
+      set_err(a.err, DEVERR_SEQ);
+      e = -1;
+    }
+    const unsigned peers = __match_any_sync(0xffffffffu, e);
+    const int rank_w = __popc(peers & ((1u << lane) - 1u));
+    if (e >= 0 && rank_w == 0) wcnt[warp][e] = __popc(peers);
+    __syncthreads();
+    for (int x = tid; x < E; x += PLAN_THREADS) {
+      int s = cnt[x];
+      for (int w = 0; w < used; ++w) {
+        const int c = wcnt[w][x];
+        wcnt[w][x] = s;
+        s += c;
+      }
+      cnt[x] = s;
+    }
+    __syncthreads();
+    if (e >= 0) a.slot_row[i] = wcnt[warp][e] + rank_w;  // rank within the expert, for now
+    else if (i < n) a.slot_row[i] = -1;
+    __syncthreads();
+  }
+  if (warp == 0) {
+    // blocks before each expert: lanes take runs of consecutive experts
+    const int per = (E + 31) / 32;
+    int mine = 0;
+    for (int j = 0; j < per; ++j) {
+      const int e = lane * per + j;
+      if (e < E) mine += (cnt[e] + 127) >> 7;
+    }
+    int end = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, end, o);
+      if (lane >= o) end += t;
+    }
+    int at = end - mine;
+    for (int j = 0; j < per; ++j) {
+      const int e = lane * per + j;
+      if (e >= E) break;
+      seg[e] = at << 7;
+      const int blocks = (cnt[e] + 127) >> 7;
+      for (int b = 0; b < blocks; ++b) a.mb_expert[at + b] = e;
+      at += blocks;
+    }
+    if (lane == 31) *a.n_mblocks = end;
+  }
+  __syncthreads();
+  for (int i = tid; i < n; i += PLAN_THREADS) {
+    const int e = a.topk_idx[i];
+    const int rk = a.slot_row[i];
+    if (rk < 0 || e < 0 || e >= E) continue;
+    const int row = seg[e] + rk;
+    a.slot_row[i] = row;
+    a.row_tok[row] = i / a.k;
+    a.row_w[row] = a.topk_w[i];
+  }
+  // padding rows of each segment
+  for (int e = warp; e < E; e += WARPS) {
+    const int pad0 = seg[e] + cnt[e], pad1 = seg[e] + (((cnt[e] + 127) >> 7) << 7);
+    for (int row = pad0 + lane; row < pad1; row += 32) {
+      a.row_tok[row] = -1;
+      a.row_w[row] = 0.f;
+    }
+  }
+  if (ROUTE && gather) {
+    __syncthreads();
+    gather_slots<T16>(a, T, ns, warp, WARPS, lane);
+  }
+}
+
+template <typename T16>
+__global__ void __launch_bounds__(256) moe_gather_kernel(MoeArgs a, int T, EpiArgs ns) {
+  grid_dep_launch();
+  grid_dep_wait();
+  gather_slots<T16>(a, T, ns, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5,
+                    threadIdx.x & 31);
 }
 
 // x[t] += sum over j of y[slot_row[t * k + j]] (j in order); with the
@@ -283,18 +329,25 @@ cudaError_t prepare_moe_kernels(int D, int E) {
   return cudaSuccess;
 }
 
-cudaError_t launch_moe_route_plan(const LaunchCtx& lc, const MoeArgs& a, int T) {
-  if (T < 1 || a.k < 1 || a.k > 8 || a.k > a.E || a.E > MOE_MAX_EXPERTS) return cudaErrorInvalidValue;
-  if (T <= FUSED_ROUTE_MAX_T) return launch_k(lc, moe_plan_kernel<true>, dim3(1), dim3(PLAN_THREADS), 0, a, T);
-  const int warps = ROUTE_THREADS / 32;
-  const size_t smem = static_cast<size_t>(warps) * a.E * 4;
-  cudaError_t e = launch_k(lc, moe_route_kernel, dim3((T + warps - 1) / warps), dim3(ROUTE_THREADS), smem, a, T);
-  if (e != cudaSuccess) return e;
-  return launch_k(lc, moe_plan_kernel<false>, dim3(1), dim3(PLAN_THREADS), 0, a, T);
-}
-
-cudaError_t launch_moe_gather(const LaunchCtx& lc, const MoeArgs& a, int T, const EpiArgs& ns) {
-  if (a.D % 8) return cudaErrorInvalidValue;
+cudaError_t launch_moe_route(const LaunchCtx& lc, const MoeArgs& a, int T, const EpiArgs& ns) {
+  if (T < 1 || a.k < 1 || a.k > 8 || a.k > a.E || a.E > MOE_MAX_EXPERTS || a.D % 8) return cudaErrorInvalidValue;
+  const bool fused = T <= FUSED_ROUTE_MAX_T;
+  const int gather = fused && T * a.k <= FUSED_GATHER_MAX ? 1 : 0;
+  cudaError_t e = cudaSuccess;
+  if (!fused) {
+    const int warps = ROUTE_THREADS / 32;
+    const size_t smem = static_cast<size_t>(warps) * a.E * 4;
+    e = launch_k(lc, moe_route_kernel, dim3((T + warps - 1) / warps), dim3(ROUTE_THREADS), smem, a, T);
+    if (e != cudaSuccess) return e;
+  }
+  const dim3 one(1), threads(PLAN_THREADS);
+  if (!fused)
+    e = launch_k(lc, moe_plan_kernel<false, bf16>, one, threads, 0, a, T, ns, gather);
+  else if (lc.f16)
+    e = launch_k(lc, moe_plan_kernel<true, f16>, one, threads, 0, a, T, ns, gather);
+  else
+    e = launch_k(lc, moe_plan_kernel<true, bf16>, one, threads, 0, a, T, ns, gather);
+  if (e != cudaSuccess || gather) return e;
   const long long warps = static_cast<long long>(T) * a.k;
   const int grid = static_cast<int>(std::min<long long>((warps + 7) / 8, 4LL * lc.num_sms));
   if (lc.f16) return launch_k(lc, moe_gather_kernel<f16>, dim3(grid), dim3(256), 0, a, T, ns);

@@ -126,10 +126,9 @@ struct MoeArgs {
   int* err;
 };
 cudaError_t prepare_moe_kernels(int D, int E);
-// Routing of T tokens from a.logits and the sorted layout (one or two launches).
-cudaError_t launch_moe_route_plan(const LaunchCtx& lc, const MoeArgs& a, int T);
-// ns: the norm state of `act` (row_rinv).
-cudaError_t launch_moe_gather(const LaunchCtx& lc, const MoeArgs& a, int T, const EpiArgs& ns);
+// Routing of T tokens from a.logits, the sorted layout and the sorted operand
+// rows (one to three launches). ns: the norm state of `act`.
+cudaError_t launch_moe_route(const LaunchCtx& lc, const MoeArgs& a, int T, const EpiArgs& ns);
 // ep: residual x (ep.x, ep.N = D) and, when ep.a_out is set, the residual
 // epilogue's outputs (a_out, a_lo_out, gain, ss_out / ss_out_stride).
 cudaError_t launch_moe_combine(const LaunchCtx& lc, const MoeArgs& a, int T, const EpiArgs& ep);
