@@ -883,7 +883,7 @@ bool persist_eligible(const axon_model* m, int B) {
 
 // Exchange buffers of the persistent step (PersistArgs::ll_*, in their order),
 // in 16-byte vectors, for PERSIST_MAX_B tokens and the widest form: a vector per
-// operand value after a residual projection or gate/up (own lines per item), a word per value
+// operand value after a residual projection (own lines per item), a word per value
 // elsewhere.
 constexpr int PERSIST_LL = 9;
 size_t persist_ll_vecs(const axon_model* m, int i) {
@@ -963,11 +963,10 @@ int enqueue_decode(axon_model* m, const int32_t* tokens, int B, int32_t* ctx, co
   int splits = m->fp32 ? 1 : attn_decode_splits(B, m->G, m->blocks_per_seq, m->num_sms, m->attn_target_ctas);
   if (splits > cap) splits = cap;
   if (persist_eligible(m, B)) {
-    // Inside one launch a cross-CTA merge costs more than it saves up to 64
-    // key blocks (8 per warp; measured at 40 blocks, head_dim 64: 0.743 ms
-    // per step unsplit, 0.775-0.790 ms split). Beyond that the keys split
-    // into items of persist_split_blocks blocks (80 blocks, head_dim 128:
-    // 3.170 ms per step in items of 16, 3.239 ms in items of 64). Head_dim
+    // Inside one launch a cross-CTA merge costs about what it saves up to 64
+    // key blocks (8 per warp; head_dim 64, unsplit / split: 0.5B width, 4 layers,
+    // 40 blocks 101.4 / 98.8 us, 135M width, short contexts 105 / 112). Beyond that
+    // the keys split into items of persist_split_blocks blocks. Head_dim
     // 128 stages one block per warp: items of 8 blocks, one round.
     const int sblocks = m->d == 128 ? 8 : m->persist_split_blocks;
     int psplits = (m->blocks_per_seq > 64 || sblocks == 8) ? (m->blocks_per_seq + sblocks - 1) / sblocks : 1;
@@ -1562,6 +1561,20 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
     m->m_head.a = m->t_a;
     ok = ok && make_tma_2d_16(&m->m_head.w, m->head, V, D, 256, m->f16);
     small_a(m->m_head, m->t_a16, m->t_a64);
+    auto mid_w = [&](GemmMaps& g, const void* w, int N, int K) {
+      ok = ok && make_tma_2d_16(&g.w192, w, N, K, 192, m->f16) && make_tma_2d_16(&g.w224, w, N, K, 224, m->f16);
+      g.mid = true;
+    };
+    for (int l = 0; l < m->L && ok; ++l) {
+      LayerW& w = m->layers[l];
+      mid_w(w.m_qkv, w.wqkv, m->Nqkv, D);
+      mid_w(w.m_o, w.wo, D, Hd);
+      if (w.Fl) {
+        mid_w(w.m_gu, w.wgu, 2 * w.Fl, D);
+        mid_w(w.m_d, w.wd, D, w.Fl);
+      }
+    }
+    mid_w(m->m_head, m->head, V, D);
     // decode projections: weight boxes of 128 rows, activation boxes of 8..64 token rows
     for (int l = 0; l < m->L && ok; ++l) {
       LayerW& w = m->layers[l];

@@ -3,8 +3,8 @@
 // activations [M][K], W = bf16 weights [N][K], fp32 accumulation in TMEM),
 // followed by the fused epilogues of epilogue.cuh.
 //
-//   warp 0      : TMA producer -- one lane streams 128x64 A and 256x64 W
-//                 tiles (128-byte swizzle) into a 4-stage shared-memory ring,
+//   warp 0      : TMA producer -- one lane streams 128x64 A and up to 256x64 W
+//                 tiles (128-byte swizzle) into a shared-memory ring,
 //                 completion tracked by mbarrier transaction bytes;
 //   warp 1      : MMA issuer -- allocates 512 TMEM columns (two 128x256 fp32
 //                 accumulators), one lane issues tcgen05.mma kind::f16
@@ -34,8 +34,8 @@ constexpr int A_BYTES = BM * BK * 2;  // 16 KB
 constexpr int EPI_WARPS = 8;
 constexpr int NUM_THREADS = 64 + 32 * EPI_WARPS;
 
-// BN_: columns of the output tile (256, or 128 where 256-wide tiles leave
-// the last wave mostly empty). SPLIT: the A operand is the sum of two
+// BN_: columns of the output tile that the ring holds (256: 256, 224 or 192 at
+// run time; or 128; gemm_tile_n chooses). SPLIT: the A operand is the sum of two
 // 16-bit terms (hi + lo) and every k-step issues two MMAs into the same
 // accumulator. The ring takes as many stages as fit in 200 KB, at most 6
 // (BN 256: 4, split 3; BN 128: 6, split 4).
@@ -87,11 +87,13 @@ AXON_DEV void tile_coords(int t, int num_m, int num_n, int& mb, int& nb) {
 template <int KIND, typename T16, bool SPLIT, int BN_, int AROWS>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                   const __grid_constant__ CUtensorMap tmAlo, int M, int N, int K, EpiArgs ep, GemmGroup grp) {
+                   const __grid_constant__ CUtensorMap tmAlo, int M, int N, int K, int width, EpiArgs ep, GemmGroup grp) {
   using C = GCfgK<KIND, SPLIT, BN_, AROWS>;
   constexpr bool SMALL = C::SMALL;
   constexpr int BN = C::BN;
   constexpr int B_BYTES = C::B_BYTES;
+  constexpr bool ANY_WIDTH = BN == 256 && !SMALL;
+  const int bn = ANY_WIDTH ? width : BN;  // columns of this launch's tiles
   constexpr uint32_t TMEM_COLS = C::TMEM_COLS;
   constexpr int STAGES = C::STAGES;
   constexpr int STAGE_BYTES = C::STAGE_BYTES;
@@ -143,7 +145,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   // grouped: the m-blocks the routing plan laid out (read after the wait,
   // when the plan kernel's writes are visible)
   const bool grouped = grp.mb_expert != nullptr;
-  const int num_m = grouped ? __ldcg(grp.n_mblocks) : (M + BM - 1) / BM, num_n = (N + BN - 1) / BN;
+  const int num_m = grouped ? __ldcg(grp.n_mblocks) : (M + BM - 1) / BM, num_n = (N + bn - 1) / bn;
   const int tiles = num_m * num_n, KB = K / BK;
 
   if (warp == 0) {
@@ -157,7 +159,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           mb = t / num_n;
           nb = t - mb * num_n;
         }
-        const int wrow = grouped ? __ldcg(grp.mb_expert + mb) * N + nb * BN : nb * BN;
+        const int wrow = grouped ? __ldcg(grp.mb_expert + mb) * N + nb * bn : nb * bn;
         for (int kb = 0; kb < KB; ++kb, ++it) {
           const int s = it % STAGES;
           const uint32_t ph = (it / STAGES) & 1;
@@ -165,7 +167,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             ok = false;
             break;
           }
-          mbar_arrive_expect_tx(full_bar(s), STAGE_BYTES);
+          mbar_arrive_expect_tx(full_bar(s), STAGE_BYTES - (BN - bn) * (BK * 2));
           tma_load_2d(a_at(s), &tmA, full_bar(s), kb * BK, mb * BM);
           if (SPLIT) tma_load_2d(alo_at(s), &tmAlo, full_bar(s), kb * BK, mb * BM);
           tma_load_2d(b_at(s), &tmB, full_bar(s), kb * BK, wrow);
@@ -175,7 +177,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     __syncwarp();
   } else if (warp == 1) {
     if (lane == 0) {
-      constexpr uint32_t idesc = idesc_f32acc(BM, BN, MmaFmt<T16>::v);
+      const uint32_t idesc = idesc_f32acc(BM, bn, MmaFmt<T16>::v);
       int it = 0, lt = 0;
       bool ok = true;
       for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++lt) {
@@ -212,8 +214,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     // two warps per TMEM lane quarter (the one that a warp may read), half the
     // tile's columns each
     const int q4 = warp & 3, half = (warp - 2) >> 2;
-    constexpr int HALF = BN / 2;
-    const int cb = half * HALF;
+    // whole groups of 32 columns: the first half takes the odd one
+    const int mid = (bn / 32 + 1) / 2 * 32;
+    const int cb = half ? mid : 0, ce = half ? bn : mid;
     const int row = q4 * 32 + lane;
     int lt = 0;
     for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++lt) {
@@ -254,7 +257,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         // one group ahead so that their round trip overlaps the previous
         // group's stores
         auto load_x = [&](int c0, float4 (&xr)[8]) {
-          const int n = nb * BN + c0 + lc;
+          const int n = nb * bn + c0 + lc;
 #pragma unroll
           for (int i = 0; i < 8; ++i)
             xr[i] = (rv[i] && n < N) ? __ldcg(reinterpret_cast<const float4*>(
@@ -267,8 +270,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         float4 xcur[8], xnext[8];
         load_x(cb, xcur);
 #pragma unroll 1
-        for (int c0 = cb; c0 < cb + HALF; c0 += 32) {
-          if (c0 + 32 < cb + HALF) load_x(c0 + 32, xnext);
+        for (int c0 = cb; c0 < ce; c0 += 32) {
+          if (c0 + 32 < ce) load_x(c0 + 32, xnext);
           uint32_t v[2][16];
           tmem_ld16(taddr + c0, v[0]);
           tmem_ld16(taddr + c0 + 16, v[1]);
@@ -279,7 +282,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 make_float4(__uint_as_float(v[j >> 2][(j & 3) * 4]), __uint_as_float(v[j >> 2][(j & 3) * 4 + 1]),
                             __uint_as_float(v[j >> 2][(j & 3) * 4 + 2]), __uint_as_float(v[j >> 2][(j & 3) * 4 + 3]));
           __syncwarp();
-          const int n = nb * BN + c0 + lc;
+          const int n = nb * bn + c0 + lc;
           const float4 g4 = n < N ? *reinterpret_cast<const float4*>(ep.gain + n) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
@@ -323,11 +326,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         }
       }
 #pragma unroll 1
-      for (int c2 = cb; c2 < cb + HALF && KIND != EPI_RESID; c2 += 32) {
+      for (int c2 = cb; c2 < ce && KIND != EPI_RESID; c2 += 32) {
         uint32_t v2[2][16];
         tmem_ld16(taddr + c2, v2[0]);
         tmem_ld16(taddr + c2 + 16, v2[1]);
-        const int n2 = nb * BN + c2;
+        const int n2 = nb * bn + c2;
         // both chunks' rotation pairs and biases are requested together
         QkvIn in[KIND == EPI_QKV ? 2 : 1];
         if (KIND == EPI_QKV && mval) {
@@ -384,8 +387,8 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 
 template <int KIND, typename T16, bool SPLIT, int BN, int AROWS>
 cudaError_t launch_kind(const LaunchCtx& lc, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
-                        const GemmGroup& grp) {
-  const int tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
+                        const GemmGroup& grp, int width) {
+  const int tiles = ((M + BM - 1) / BM) * ((N + width - 1) / width);
   // grouped: the tile count is known only on the device; one CTA per SM
   const int grid = grp.mb_expert ? lc.num_sms : (tiles < lc.num_sms ? tiles : lc.num_sms);
   cudaLaunchConfig_t cfg = {};
@@ -400,8 +403,9 @@ cudaError_t launch_kind(const LaunchCtx& lc, const GemmMaps& maps, int M, int N,
   cfg.numAttrs = lc.pdl ? 1 : 0;
   const GemmMaps& g = BN == 256 ? maps : *maps.n128;
   const CUtensorMap& ta = AROWS == 16 ? g.a16 : (AROWS == 64 ? g.a64 : g.a);
+  const CUtensorMap& w = width == 224 ? g.w224 : (width == 192 ? g.w192 : g.w);
   const CUtensorMap& tlo = SPLIT ? (AROWS == 16 ? g.a_lo16 : (AROWS == 64 ? g.a_lo64 : g.a_lo)) : ta;
-  return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<KIND, T16, SPLIT, BN, AROWS>, ta, g.w, tlo, M, N, K, ep, grp);
+  return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<KIND, T16, SPLIT, BN, AROWS>, ta, w, tlo, M, N, K, width, ep, grp);
 }
 
 }  // namespace
@@ -475,42 +479,52 @@ cudaError_t prepare_gemm_t() {
 }
 template <typename T16, int BN, int AROWS>
 cudaError_t launch_t(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
-                     const GemmGroup& grp) {
+                     const GemmGroup& grp, int width) {
   switch (kind) {
     case EPI_QKV:
-      return maps.split ? launch_kind<EPI_QKV, T16, true, BN, AROWS>(lc, maps, M, N, K, ep, grp)
-                        : launch_kind<EPI_QKV, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, grp);
-    case EPI_RESID: return launch_kind<EPI_RESID, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, grp);
-    case EPI_SWIGLU: return launch_kind<EPI_SWIGLU, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, grp);
-    case EPI_ROWSCALE: return launch_kind<EPI_ROWSCALE, T16, false, BN, 128>(lc, maps, M, N, K, ep, grp);
-    default: return launch_kind<EPI_LOGITS, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, grp);
+      return maps.split ? launch_kind<EPI_QKV, T16, true, BN, AROWS>(lc, maps, M, N, K, ep, grp, width)
+                        : launch_kind<EPI_QKV, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, grp, width);
+    case EPI_RESID: return launch_kind<EPI_RESID, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, grp, width);
+    case EPI_SWIGLU: return launch_kind<EPI_SWIGLU, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, grp, width);
+    case EPI_ROWSCALE: return launch_kind<EPI_ROWSCALE, T16, false, BN, 128>(lc, maps, M, N, K, ep, grp, width);
+    default: return launch_kind<EPI_LOGITS, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, grp, width);
   }
 }
 template <int BN, int AROWS>
 cudaError_t launch_ar(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
-                      const GemmGroup& grp) {
-  return lc.f16 ? launch_t<f16, BN, AROWS>(lc, kind, maps, M, N, K, ep, grp)
-                : launch_t<bf16, BN, AROWS>(lc, kind, maps, M, N, K, ep, grp);
+                      const GemmGroup& grp, int width) {
+  return lc.f16 ? launch_t<f16, BN, AROWS>(lc, kind, maps, M, N, K, ep, grp, width)
+                : launch_t<bf16, BN, AROWS>(lc, kind, maps, M, N, K, ep, grp, width);
 }
 template <int BN>
 cudaError_t launch_bn(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
-                      const GemmGroup& grp, int arows) {
-  if (arows == 16) return launch_ar<BN, 16>(lc, kind, maps, M, N, K, ep, grp);
-  if (arows == 64) return launch_ar<BN, 64>(lc, kind, maps, M, N, K, ep, grp);
-  return launch_ar<BN, 128>(lc, kind, maps, M, N, K, ep, grp);
+                      const GemmGroup& grp, int arows, int width) {
+  if (arows == 16) return launch_ar<BN, 16>(lc, kind, maps, M, N, K, ep, grp, width);
+  if (arows == 64) return launch_ar<BN, 64>(lc, kind, maps, M, N, K, ep, grp, width);
+  return launch_ar<BN, 128>(lc, kind, maps, M, N, K, ep, grp, width);
 }
 }  // namespace
 
-// Output-tile width for an M x N product: 128 where 256-wide tiles leave
-// the last wave mostly idle (cost in column-waves: waves x width, plus a
-// per-tile overhead worth 16 columns), 256 otherwise.
+// Output-tile width for an M x N product: the cheapest count of waves, each
+// priced by its width. A wave costs less than its columns: at 128 the
+// reads of A weigh more and the tensor cores idle (down projection of 8B width,
+// a wave of 128 / 192 / 224 / 256 columns 63 / 83.5 / 89 / 92 us: the weights
+// below). 192 and 224 fill waves that the others leave half empty (8B width, 1024
+// rows: QKV 128 62.7 us, 192 54.4, 256 59.0; down 256 92.0, 224 89.4; 1300 rows: O 128
+// 63.5, 192 54.7, 256 60.1; down 186 / 157 / 167; 32B width, 512 rows: O 256 46.9, 192
+// 40.8; 1024 rows: down 128 348, 192 283, 256 303). At most 64 rows (the small-M
+// stages) and the grouped products know 128 and 256 only: 128 where 256-wide tiles
+// leave the last wave mostly idle.
 int gemm_tile_n(const LaunchCtx& lc, const GemmMaps& maps, int M, int N) {
   if (!maps.n128) return 256;
   const long long mt = (M + BM - 1) / BM;
-  const long long t256 = mt * ((N + 255) / 256), t128 = mt * ((N + 127) / 128);
-  const long long w256 = (t256 + lc.num_sms - 1) / lc.num_sms, w128 = (t128 + lc.num_sms - 1) / lc.num_sms;
-  const long long c256 = w256 * (256 + 16), c128 = w128 * (128 + 16);
-  return c128 * 100 < c256 * 85 ? 128 : 256;
+  auto waves = [&](int bn) { return (mt * ((N + bn - 1) / bn) + lc.num_sms - 1) / lc.num_sms; };
+  if (!maps.mid || M <= 64) return waves(128) * (128 + 16) * 100 < waves(256) * (256 + 16) * 85 ? 128 : 256;
+  constexpr int WIDTH[4] = {256, 224, 192, 128}, COST[4] = {146, 139, 132, 100};
+  int best = 0;
+  for (int i = 1; i < 4; ++i)
+    if (waves(WIDTH[i]) * COST[i] < waves(WIDTH[best]) * COST[best]) best = i;
+  return WIDTH[best];
 }
 
 cudaError_t prepare_gemm_kernels() {
@@ -529,9 +543,11 @@ cudaError_t launch_gemm_tc(const LaunchCtx& lc, int kind, const GemmMaps& maps, 
   // rows: the small-M stage layouts
   const bool dec = !grp.mb_expert && kind != EPI_ROWSCALE;
   const int arows = (dec && M <= 16 && maps.has16) ? 16 : ((dec && M <= 64 && maps.has64) ? 64 : 128);
+  const bool mid = maps.mid && arows == 128 && !grp.mb_expert;
+  if (tile_n != 256 && tile_n != 128 && !(mid && (tile_n == 192 || tile_n == 224))) return cudaErrorInvalidValue;
   if (tile_n == 128) {
     if (!maps.n128) return cudaErrorInvalidValue;
-    return launch_bn<128>(lc, kind, maps, M, N, K, ep, grp, arows);
+    return launch_bn<128>(lc, kind, maps, M, N, K, ep, grp, arows, 128);
   }
-  return launch_bn<256>(lc, kind, maps, M, N, K, ep, grp, arows);
+  return launch_bn<256>(lc, kind, maps, M, N, K, ep, grp, arows, tile_n);
 }

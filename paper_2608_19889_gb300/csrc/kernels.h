@@ -198,6 +198,8 @@ cudaError_t prepare_gemm_kernels();
 struct GemmMaps {
   CUtensorMap a;     // activations [rows][K], box 64 x 128
   CUtensorMap w;     // weights [N][K], box 64 x 256 (64 x 128 in the n128 set)
+  CUtensorMap w192;  // the same weights in boxes of 192 and 224 rows (when mid)
+  CUtensorMap w224;
   CUtensorMap a_lo;  // second term of a split activation operand (used when split)
   // the same activation operand (and second term) in boxes of 16 and of 64
   // rows: at most 16 (64) rows (decode), the ring stages hold only those
@@ -208,6 +210,7 @@ struct GemmMaps {
   bool has16 = false;
   bool has64 = false;
   bool split = false;
+  bool mid = false;
   const GemmMaps* n128 = nullptr;  // the same operands with 128-row weight boxes (128-wide tiles), or null
 };
 bool make_tma_2d_16(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, bool f16);
@@ -230,7 +233,7 @@ struct GemmGroup {
   const int* n_mblocks = nullptr;
   const int* row_valid = nullptr;
 };
-// tile_n: 256 or 128 (from gemm_tile_n); the residual epilogue writes two
+// tile_n: 256, 224, 192 or 128 (from gemm_tile_n); the residual epilogue writes two
 // norm partials per row and tile, i.e. 2 * ceil(N / tile_n) of them.
 cudaError_t launch_gemm_tc(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
                            int tile_n = 256, const GemmGroup* group = nullptr);
