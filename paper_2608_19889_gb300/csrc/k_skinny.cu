@@ -14,10 +14,10 @@
 //
 // Measured against the kernels that it replaced (the GEMV up to 32 tokens, split-K
 // GEMM through L2, unsplit GEMM): 8B width, 64 tokens in fp16, one layer over a paged
-// cache 309 -> 229 us of which the attention takes 103 (QKV 36.9 -> 20 us, O 29 ->
-// 13, gate/up 50 -> 40 (235 MB), down 53 -> 29 (117 MB)); 32B width, 16 tokens, one
-// layer 253 -> 224 us. About 5 us of each launch are fixed: launch, first weights,
-// cluster barrier, epilogue.
+// cache 308 -> 229 us of which the attention takes 99 (QKV 36.9 -> 20.3 us, O 29 ->
+// 15.2, gate/up 50 -> 43.4 (235 MB), down 53 -> 28.4 (117 MB)); 32B width, 16 tokens,
+// one layer 253 -> 222 us. About 5 us of each launch are fixed: launch, first
+// weights, cluster barrier, epilogue.
 //
 //   warp 0 : TMA producer; requests the first stages' weights before the
 //            preceding kernel has finished (they depend on nothing);
