@@ -107,7 +107,6 @@ struct axon_model {
   void* a_lo_last = nullptr;  // fp16 mode
   float* rinv_last = nullptr;  // [max_batch]
   SplitKWork splitk{};     // decode projections' cross-CTA split-K workspace
-  int* ticket = nullptr;   // last-CTA counter of the residual producers
   float* attn_part = nullptr;
   int* attn_cnt = nullptr;
   int max_splits = 1;
@@ -494,19 +493,19 @@ inline void pend(Prof* p, double bytes, double flops) {
 //   8B width, 2 layers: 4 tokens (qk-norm) 220 / 204, 8 tokens 234 / 210, prompt of
 //     2 tokens 232 / 199, of 64 (fp16) 817 / 245; 32B width, 1 layer, 2 tokens
 //     196 / 193, 8 tokens 206 / 195;
-//   16B mixture of experts, 2 layers (O projection 2048 x 2048): 1 token 169 / 174,
-//     8 tokens 253 / 252, 12 tokens 308 / 294, prompt of 4 tokens 204 / 210, of 9
-//     247 / 241, of 32 349 / 298;
-//   0.5B width, 4 layers: 9 tokens 178 / 164, 24 tokens 218 / 172, prompt of 9
-//     tokens 153 / 155, of 16 160 / 157, of 64 238 / 210;
-//   135M width, 6 layers: 9 tokens 180 / 189 (fp16 210 / 203), 16 tokens 192 / 193, 24
-//     tokens 232 / 198, prompt of 16 tokens 168 / 183, of 32 227 / 197.
-int tc_min_rows(const axon_model* m) {
+//   16B mixture of experts, 2 layers (O projection 2048 x 2048): 1 token 154 / 166,
+//     5 tokens 215 / 221, 8 tokens 240 / 242 (fp16 253 / 256), 9 tokens 261 / 252, 12
+//     tokens 295 / 283, prompt of 4 tokens 189 / 202, of 9 232 / 231, of 16 360 / 248;
+//   0.5B width, 4 layers: 9 tokens 170 / 164 (fp16 195 / 177), 16 tokens 180 / 165, prompt of
+//     9 tokens 145 / 154 (fp16 163 / 164), of 16 153 / 157 (171 / 168), of 32 195 / 172;
+//   135M width, 6 layers: 9 tokens 165 / 189 (fp16 194 / 203), 16 tokens 177 / 193 (213 /
+//     208), 17 tokens 208 / 196, prompt of 16 tokens 147 / 183 (168 / 195), of 32 206 / 197.
+int tc_min_rows(const axon_model* m, bool decode) {
   const long long small =  // weights of the smaller attention projection
       std::min(static_cast<long long>(m->Nqkv) * m->D, static_cast<long long>(m->D) * m->H * m->d);
   if (small >= 1 << 23) return 1;
-  if (small >= 1 << 21) return 5;
-  return m->f16 || 2LL * m->F * m->D >= 1 << 21 ? 9 : 17;
+  if (small >= 1 << 21) return 9;
+  return (decode || m->f16) && 2LL * m->F * m->D >= 1 << 21 ? 9 : 17;
 }
 
 // One projection: picks the kernel for the mode and row count.
@@ -531,11 +530,6 @@ struct Proj {
       else if (decode && act == m->u) lo = m->u_lo;
     }
     if (!tc && (M <= 64 || (!m->fp32 && maps == nullptr))) {
-      if (kind == EPI_RESID) {
-        ep.rinv_out = m->rinv;
-        ep.ticket = m->ticket;
-        ns.rinv = true;
-      }
       rc = launch_gemv(lc, kind, m->fp32, W, N, K, act, act_stride, M, ep, m->splitk, lo);
       ns.parts = N / 16;
       return ns;
@@ -739,7 +733,7 @@ bool attn_on_tcgen05(int M, int S, bool varlen) {
 int enqueue_prefill(axon_model* m, const int32_t* ids, int B, int S, const int32_t* bt, int logits_mode, float* logits,
                     int32_t* next, cudaStream_t st, Prof* pf = nullptr, const VarlenBatch* vl = nullptr) {
   const int M = vl ? vl->T : B * S;
-  const bool tc = !m->fp32 && (M > 64 || M >= tc_min_rows(m));
+  const bool tc = !m->fp32 && (M > 64 || M >= tc_min_rows(m, false));
   LaunchCtx lc{st, m->use_pdl && !pf, m->num_sms, m->f16};
   const int2* rowmap = vl ? m->rowmap : nullptr;
   if (vl) CK(launch_varlen_rows(lc, vl->cu, vl->ctx, B, M, vl->max_chunk, m->cfg.max_context, m->rowmap, m->err));
@@ -942,7 +936,7 @@ PersistArgs persist_args(const axon_model* m, const int32_t* tokens, int B, int3
 int enqueue_decode(axon_model* m, const int32_t* tokens, int B, int32_t* ctx, const int32_t* bt, float* logits,
                    int32_t* next, cudaStream_t st, Prof* pf = nullptr, double kv_tokens = 0,
                    float* attn_part = nullptr, int* attn_cnt = nullptr, int attn_rows_cap = 0) {
-  const bool tc = !m->fp32 && B >= tc_min_rows(m);
+  const bool tc = !m->fp32 && B >= tc_min_rows(m, true);
   LaunchCtx lc{st, m->use_pdl && !pf, m->num_sms, m->f16, tc ? 100 : -1};
   g_trace_stream = st;
   Proj pj{m, lc};
@@ -1453,8 +1447,6 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
   if (m->f16 && (rc = dev_alloc(m, &m->a_lo_last, static_cast<size_t>(cfg->max_batch) * D * es))) return fail(rc);
   if ((rc = dev_alloc(m, &p, static_cast<size_t>(cfg->max_batch) * 4))) return fail(rc);
   m->rinv_last = static_cast<float*>(p);
-  if ((rc = dev_alloc(m, &p, 16))) return fail(rc);
-  m->ticket = static_cast<int*>(p);
   m->splitk.max_tiles = 1024;
   m->splitk.max_ctas = 2048;
   if ((rc = dev_alloc(m, &p, static_cast<size_t>(m->splitk.max_ctas) * 16 * 64 * 4))) return fail(rc);
@@ -1473,7 +1465,7 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
   m->err = static_cast<int*>(p);
   if (cudaMemsetAsync(m->keys, 0, static_cast<size_t>(Mcap) * 8, st) != cudaSuccess ||
       cudaMemsetAsync(m->attn_cnt, 0, static_cast<size_t>(dec_b) * m->G * 4, st) != cudaSuccess ||
-      cudaMemsetAsync(m->err, 0, 16, st) != cudaSuccess || cudaMemsetAsync(m->ticket, 0, 16, st) != cudaSuccess ||
+      cudaMemsetAsync(m->err, 0, 16, st) != cudaSuccess ||
       cudaMemsetAsync(m->x, 0, static_cast<size_t>(Mcap) * D * 4, st) != cudaSuccess ||
       cudaMemsetAsync(m->a, 0, static_cast<size_t>(Mcap) * D * es, st) != cudaSuccess ||
       cudaMemsetAsync(m->o, 0, static_cast<size_t>(Mcap) * Hd * es, st) != cudaSuccess ||

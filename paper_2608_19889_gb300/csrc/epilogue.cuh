@@ -69,10 +69,6 @@ struct EpiArgs {
   const float* gain;   // [N]
   float* ss_out;       // [M][ss_out_stride]
   int ss_out_stride;
-  // Decode projections: the last CTA to finish reduces the partials into
-  // rinv_out[m] (ticket: a zeroed counter it resets).
-  float* rinv_out;
-  int* ticket;
   // SWIGLU
   void* u_out;     // [M][N/2]
   void* u_lo_out;  // optional [M][N/2]: u - u_out (second term of the down projection's operand)
