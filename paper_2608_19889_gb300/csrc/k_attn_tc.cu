@@ -15,20 +15,29 @@
 //   warp 9           : MMA issuer -- S = Q K^T into TMEM, O += P V with P
 //                      read back from TMEM and O accumulating in TMEM.
 // The 512 TMEM columns hold S0, S1 (128 each) and O0, O1 (HD each); a tile's
-// probabilities (16-bit, 64 columns) overwrite its scores. The issuer alternates
-// the tiles, so one tile's softmax runs under the other's MMAs.
+// probabilities (16-bit, 64 columns) and their second terms (8 columns) overwrite
+// its scores. The issuer alternates the tiles, so one tile's softmax runs under the
+// other's MMAs.
 //
-// The output is rescaled in TMEM only when a row's maximum grew by more than
-// 2^8 since the last rescale (probabilities then reach at most 2^8, far inside
-// both 16-bit ranges, and are rounded to the same relative precision); the
-// rescale factor is exact in the sense of the online softmax.
+// Rounding of the probabilities, which must cost no more than in the mma.sync
+// kernel: O is rescaled in TMEM whenever a row's maximum has grown, so that the
+// largest probability is 1 and enters P V exactly; the row sum takes the rounded
+// values; and since a maximum over 128 keys leaves fewer of a row's running
+// maxima exact than one over 32, the first KT2 keys of a tile have a second 16-bit
+// term (one more MMA of 16 keys). rms error of one layer in fp16, this / mma.sync, at
+// scores of standard deviation 1.0, 1.64 (8B width) and 2.5: 0.982, 0.992, 0.994; without
+// the second terms 1.010, 1.012, 1.005; rescaled only on a growth of 2^8 and with an
+// unrounded sum 1.059, 1.103, 1.147; with second terms of all keys 0.789, 0.857, 0.913 at
+// 22 % more time. Whole prefills against 64 bits, 8B width, fp16, 512 tokens: mma.sync 8.53e-4,
+// this 8.50e-4 (rescaled on 2^8: 8.65e-4).
 //
-// Bound: at head_dim 128 a 128 x 128 tile takes 512 tensor cycles and as many
+// Bound: at head_dim 128 a 128 x 128 tile takes 544 tensor cycles and nearly as many
 // exponential-unit cycles, and the softmax's issue slots come to about the
-// same. Measured against the mma.sync kernel (4 warps x 16 rows, scores in
-// registers, k_attn.cu; still taken for short prompts): 8B width, 8191 positions
-// under a 4096-key window 1677 -> 338 us (246 -> 1220 TFLOP/s), 32B width,
-// 4 x 2048 positions 844 -> 212 us, 8B width, 1024 positions 59.5 -> 25.4 us.
+// same. Measured by events against the mma.sync kernel (4 warps x 16 rows, scores in
+// registers, k_attn.cu; still taken for short prompts) and this one with the lagging
+// maximum: 8B width, 8191 positions under a 4096-key window 1681 / 387 / 432 us,
+// 32B width, 4 x 2048 positions 916 / 243 / 269 us, 8B width, 1024 positions
+// 62 / 28.8 / 30.9 us.
 #include <math.h>
 
 #include "kernels.h"
@@ -37,7 +46,7 @@ namespace {
 
 constexpr int TC_THREADS = 320;
 constexpr int KT = 128;  // keys per tile
-constexpr float RESCALE_LOG2 = 8.f;
+constexpr int KT2 = 16;  // the first keys of a tile: their probabilities have two 16-bit terms
 
 template <int HD>
 struct ACfg {
@@ -89,6 +98,11 @@ AXON_DEV void tmem_st32(uint32_t taddr, const uint32_t* r) {
       "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
       : "memory");
 }
+AXON_DEV void tmem_st8(uint32_t taddr, const uint32_t* r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]),
+               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
 AXON_DEV void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 AXON_DEV float ex2(float v) {
@@ -109,17 +123,38 @@ AXON_DEV uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
 }
-AXON_DEV uint64_t add2(uint64_t a, uint64_t b) {
+AXON_DEV uint64_t mul2(uint64_t a, uint64_t b) {
   uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
-// Probabilities lie in [0, 2^RESCALE_LOG2]: no saturation needed.
+// Probabilities lie in [0, 1]: no saturation needed.
 template <typename T> AXON_DEV uint32_t pack_p(float lo, float hi);
 template <> AXON_DEV uint32_t pack_p<bf16>(float lo, float hi) { return pack_bf2(lo, hi); }
 template <> AXON_DEV uint32_t pack_p<f16>(float lo, float hi) {
   __half2 h = __floats2half2_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&h);
+}
+// What the two 16-bit roundings in p lost of a and e.
+template <typename T> AXON_DEV uint32_t pack_rest(float a, float e, uint32_t p);
+template <> AXON_DEV uint32_t pack_rest<bf16>(float a, float e, uint32_t p) {
+  return pack_bf2(a - bf_lo(p), e - bf_hi(p));
+}
+template <> AXON_DEV uint32_t pack_rest<f16>(float a, float e, uint32_t p) {
+  const float2 r = __half22float2(*reinterpret_cast<__half2*>(&p));
+  return pack_p<f16>(a - r.x, e - r.y);
+}
+// lo += the low, hi += the high 16-bit value of p.
+template <typename T> AXON_DEV void add_p(float& lo, float& hi, uint32_t p);
+template <> AXON_DEV void add_p<bf16>(float& lo, float& hi, uint32_t p) {
+  asm("{\n .reg .b16 l, h;\n mov.b32 {l, h}, %2;\n add.f32.bf16 %0, l, %0;\n add.f32.bf16 %1, h, %1;\n}"
+      : "+f"(lo), "+f"(hi)
+      : "r"(p));
+}
+template <> AXON_DEV void add_p<f16>(float& lo, float& hi, uint32_t p) {
+  asm("{\n .reg .f16 l, h;\n mov.b32 {l, h}, %2;\n add.f32.f16 %0, l, %0;\n add.f32.f16 %1, h, %1;\n}"
+      : "+f"(lo), "+f"(hi)
+      : "r"(p));
 }
 
 // The V tile as the B operand of P V: N = dims (contiguous in memory), K =
@@ -322,9 +357,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
           if (!ok) break;
           tc_fence_after();
           const int ks = more ? KT / 16 : tail / 16;
-          for (int k = 0; k < ks; ++k)
-            tc_mma_f16_ts(tmem + 2 * KT + w * HD, tmem + w * KT + k * 8, v_desc<HD>(sKV + sv * C::TILE + k * 2048),
-                          id_o, (t != 0 || k != 0) ? 1u : 0u);
+          for (int k = 0; k < ks; ++k) {
+            const uint64_t vd = v_desc<HD>(sKV + sv * C::TILE + k * 2048);
+            tc_mma_f16_ts(tmem + 2 * KT + w * HD, tmem + w * KT + k * 8, vd, id_o, (t != 0 || k != 0) ? 1u : 0u);
+            if (k < KT2 / 16) tc_mma_f16_ts(tmem + 2 * KT + w * HD, tmem + w * KT + KT / 2 + k * 8, vd, id_o, 1u);
+          }
           // MMAs run in issue order: the next scores may overwrite the
           // probabilities just issued, and s_full implies that O is up to date
           if (more)
@@ -387,48 +424,53 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             mx[u] = c + 4 + u < KT ? fmaxf(mx[u], fmaxf(s[c + u], s[c + 4 + u])) : fmaxf(mx[u], s[c + u]);
         }
         const float mt = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sl2;
-        // -inf + 8 is -inf: the first finite maximum always counts as grown
-        if (__any_sync(0xffffffffu, mt > m + RESCALE_LOG2)) {
+        if (__any_sync(0xffffffffu, mt > m)) {
           const float nm = fmaxf(m, mt);
           const float f = m == -INFINITY ? 0.f : ex2(m - nm);
           l *= f;
           m = nm;
           if (t > 0) {
+            const uint64_t f2 = pk2(f, f);
 #pragma unroll 1
             for (int c = 0; c < HD; c += 32) {
-              uint32_t o[32];
-              tmem_ld32(tO + c, o);
+              float o[32];
+              tmem_ld32(tO + c, reinterpret_cast<uint32_t*>(o));
               tmem_wait_ld();
 #pragma unroll
-              for (int u = 0; u < 32; ++u) o[u] = __float_as_uint(__uint_as_float(o[u]) * f);
-              tmem_st32(tO + c, o);
+              for (int u = 0; u < 32; u += 2) upk2(mul2(pk2(o[u], o[u + 1]), f2), o[u], o[u + 1]);
+              tmem_st32(tO + c, reinterpret_cast<uint32_t*>(o));
             }
           }
         }
         const float nb = m == -INFINITY ? 0.f : -m;
         const uint64_t sl2p = pk2(sl2, sl2), nbp = pk2(nb, nb);
-        uint64_t sum[2] = {0ull, 0ull};
+        float sum[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int c0 = 0; c0 < KT; c0 += 64) {
           if (c0 == 64 && half) break;
-          uint32_t pr[32];
+          uint32_t pr[32], rest[8];
 #pragma unroll
           for (int c = 0; c < 32; ++c) {
             float a, e;
             upk2(fma2(pk2(s[c0 + 2 * c], s[c0 + 2 * c + 1]), sl2p, nbp), a, e);
             a = ex2(a);
             e = ex2(e);
-            sum[c & 1] = add2(sum[c & 1], pk2(a, e));
             pr[c] = pack_p<T16>(a, e);
+            if (c0 == 0 && c < KT2 / 2) {
+              rest[c & 7] = pack_rest<T16>(a, e, pr[c]);
+              sum[(c & 1) * 2] += a;
+              sum[(c & 1) * 2 + 1] += e;
+              if ((c & 7) == 7) tmem_st8(tS + KT / 2 + (c & ~7), rest);
+            } else {
+              add_p<T16>(sum[(c & 1) * 2], sum[(c & 1) * 2 + 1], pr[c]);
+            }
           }
           tmem_st32(tS + c0 / 2, pr);
         }
         tmem_wait_st();
         tc_fence_before();
         mbar_arrive(p_full(w));
-        float a, e;
-        upk2(add2(sum[0], sum[1]), a, e);
-        l += a + e;
+        l += (sum[0] + sum[1]) + (sum[2] + sum[3]);
       }
       if (ok) ok = __all_sync(0xffffffffu, mbar_wait(o_full(w), 0, p.err));
       if (ok) {
