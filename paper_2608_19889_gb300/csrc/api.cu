@@ -500,6 +500,9 @@ inline void pend(Prof* p, double bytes, double flops) {
 //     9 tokens 145 / 154 (fp16 163 / 164), of 16 153 / 157 (171 / 168), of 32 195 / 172;
 //   135M width, 6 layers: 9 tokens 165 / 189 (fp16 194 / 203), 16 tokens 177 / 193 (213 /
 //     208), 17 tokens 208 / 196, prompt of 16 tokens 147 / 183 (168 / 195), of 32 206 / 197.
+// With the whole vocabulary and both terms of every fp16 operand: 32B width, 1 layer, 1 token
+// 454 / 445, 8 tokens 495 / 450; 8B width, 2 layers (of 32), 2 tokens 384 / 388, 3 tokens 390 / 387, 8
+// tokens 420 / 396, of which a layer at 2 tokens 8 us less on tcgen05 and the head 20 more.
 int tc_min_rows(const axon_model* m, bool decode) {
   const long long small =  // weights of the smaller attention projection
       std::min(static_cast<long long>(m->Nqkv) * m->D, static_cast<long long>(m->D) * m->H * m->d);
@@ -542,7 +545,11 @@ struct Proj {
     }
     // up to 128 rows: weights as the wide operand, K split over a cluster,
     // unless the tiles alone fill the GPU more than twice. Two terms up to 32
-    // rows (64 in a prefill), and always where the operand is split (QKV).
+    // rows (64 in a prefill), and always where the operand is split (QKV);
+    // up to 8 rows (64 in a prefill) where the tiles do fill it and the GEMM takes the
+    // product (decode step of 8 tokens, fp16, whole vocabulary, GEMV with both terms / GEMM
+    // with both / with one: 8B width, 2 layers, 415 / 396 / 377 us; 32B width, 1 layer, 480 / 450 /
+    // 426; the logits' error of a lost term 2e-4 against 7e-6).
     // Residual projections of more rows too while few tiles share a long K
     // (whole passes, tcgen05 GEMM / this: 0.5B width, 4 layers, prompts of 129,
     // 512, 1000 tokens 260 / 237, 314 / 293, 367 / 362 us; 8B width, 2 layers, 160
@@ -561,7 +568,8 @@ struct Proj {
       }
     }
     const int tn = gemm_tile_n(lc, *maps, M, N);
-    rc = launch_gemm_tc(lc, kind, *maps, M, N, K, ep, tn);
+    const bool gemm_lo = lo != nullptr && maps->has_lo && (kind == EPI_SWIGLU || kind == EPI_LOGITS) && M <= (decode ? 8 : 64);
+    rc = launch_gemm_tc(lc, kind, *maps, M, N, K, ep, tn, nullptr, gemm_lo);
     ns.parts = 2 * ((N + tn - 1) / tn);
     return ns;
   }
@@ -1494,12 +1502,14 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
     for (const LayerW& w : m->layers)
       if (w.Fl && !m->am_u.count(w.Fl))
         ok = ok && make_act_maps(&m->am_u[w.Fl], m->u, m->u_lo, Mcap, m->cfg.max_batch, w.Fl, m->f16);
-    auto small_a = [&](GemmMaps& g, const CUtensorMap& a16, const CUtensorMap& a64) {
+    // lo: the operand is `a`, which has a second term in fp16 mode
+    auto small_a = [&](GemmMaps& g, const CUtensorMap& a16, const CUtensorMap& a64, bool lo) {
       g.a16 = a16;
       g.a64 = a64;
-      if (g.split) {
+      if (lo && m->a_lo) {
         g.a_lo16 = m->t_alo16;
         g.a_lo64 = m->t_alo64;
+        g.has_lo = true;
       }
       g.has16 = g.has64 = true;
     };
@@ -1513,19 +1523,19 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
       }
       w.m_o.a = m->t_o;
       ok = ok && make_tma_2d_16(&w.m_o.w, w.wo, D, Hd, 256, m->f16);
-      small_a(w.m_qkv, m->t_a16, m->t_a64);
-      small_a(w.m_o, m->t_o16, m->t_o64);
+      small_a(w.m_qkv, m->t_a16, m->t_a64, true);
+      small_a(w.m_o, m->t_o16, m->t_o64, false);
       if (w.Fl) {
         w.m_gu.a = m->t_a;
         ok = ok && make_tma_2d_16(&w.m_gu.w, w.wgu, 2 * w.Fl, D, 256, m->f16);
         // the down projection reads u with this layer's row stride
         ok = ok && make_tma_2d_16(&w.m_d.a, m->u, Mcap, w.Fl, 128, m->f16);
         ok = ok && make_tma_2d_16(&w.m_d.w, w.wd, D, w.Fl, 256, m->f16);
-        small_a(w.m_gu, m->t_a16, m->t_a64);
+        small_a(w.m_gu, m->t_a16, m->t_a64, true);
         CUtensorMap u16, u64;
         ok = ok && make_tma_2d_16(&u16, m->u, Mcap, w.Fl, 16, m->f16) &&
              make_tma_2d_16(&u64, m->u, Mcap, w.Fl, 64, m->f16);
-        small_a(w.m_d, u16, u64);
+        small_a(w.m_d, u16, u64, false);
       }
       if (w.moe) {
         const int E = m->E, Fe = m->Fe;
@@ -1552,7 +1562,7 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
     }
     m->m_head.a = m->t_a;
     ok = ok && make_tma_2d_16(&m->m_head.w, m->head, V, D, 256, m->f16);
-    small_a(m->m_head, m->t_a16, m->t_a64);
+    small_a(m->m_head, m->t_a16, m->t_a64, true);
     auto mid_w = [&](GemmMaps& g, const void* w, int N, int K) {
       ok = ok && make_tma_2d_16(&g.w192, w, N, K, 192, m->f16) && make_tma_2d_16(&g.w224, w, N, K, 224, m->f16);
       g.mid = true;

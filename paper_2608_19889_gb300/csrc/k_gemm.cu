@@ -27,6 +27,8 @@
 
 #include <cudaTypedefs.h>
 
+#include <type_traits>
+
 namespace {
 
 constexpr int BM = 128, BK = 64, GROUP_M = 8;
@@ -467,6 +469,15 @@ cudaError_t set_smem() {
   }
   return e;
 }
+// The small-M layouts of a two-term operand (fp16 mode), beside QKV's.
+template <int KIND>
+cudaError_t set_smem_lo() {
+  cudaError_t e = set_smem1<KIND, f16, true, 256, 16>();
+  if (e == cudaSuccess) e = set_smem1<KIND, f16, true, 128, 16>();
+  if (e == cudaSuccess) e = set_smem1<KIND, f16, true, 256, 64>();
+  if (e == cudaSuccess) e = set_smem1<KIND, f16, true, 128, 64>();
+  return e;
+}
 template <typename T16>
 cudaError_t prepare_gemm_t() {
   cudaError_t e = set_smem<EPI_QKV, T16, false>();
@@ -479,7 +490,11 @@ cudaError_t prepare_gemm_t() {
 }
 template <typename T16, int BN, int AROWS>
 cudaError_t launch_t(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
-                     const GemmGroup& grp, int width) {
+                     const GemmGroup& grp, int width, bool lo) {
+  if constexpr (AROWS < BM && std::is_same<T16, f16>::value) {
+    if (lo && kind == EPI_SWIGLU) return launch_kind<EPI_SWIGLU, T16, true, BN, AROWS>(lc, maps, M, N, K, ep, grp, width);
+    if (lo && kind == EPI_LOGITS) return launch_kind<EPI_LOGITS, T16, true, BN, AROWS>(lc, maps, M, N, K, ep, grp, width);
+  }
   switch (kind) {
     case EPI_QKV:
       return maps.split ? launch_kind<EPI_QKV, T16, true, BN, AROWS>(lc, maps, M, N, K, ep, grp, width)
@@ -492,16 +507,16 @@ cudaError_t launch_t(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M,
 }
 template <int BN, int AROWS>
 cudaError_t launch_ar(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
-                      const GemmGroup& grp, int width) {
-  return lc.f16 ? launch_t<f16, BN, AROWS>(lc, kind, maps, M, N, K, ep, grp, width)
-                : launch_t<bf16, BN, AROWS>(lc, kind, maps, M, N, K, ep, grp, width);
+                      const GemmGroup& grp, int width, bool lo) {
+  return lc.f16 ? launch_t<f16, BN, AROWS>(lc, kind, maps, M, N, K, ep, grp, width, lo)
+                : launch_t<bf16, BN, AROWS>(lc, kind, maps, M, N, K, ep, grp, width, lo);
 }
 template <int BN>
 cudaError_t launch_bn(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
-                      const GemmGroup& grp, int arows, int width) {
-  if (arows == 16) return launch_ar<BN, 16>(lc, kind, maps, M, N, K, ep, grp, width);
-  if (arows == 64) return launch_ar<BN, 64>(lc, kind, maps, M, N, K, ep, grp, width);
-  return launch_ar<BN, 128>(lc, kind, maps, M, N, K, ep, grp, width);
+                      const GemmGroup& grp, int arows, int width, bool lo) {
+  if (arows == 16) return launch_ar<BN, 16>(lc, kind, maps, M, N, K, ep, grp, width, lo);
+  if (arows == 64) return launch_ar<BN, 64>(lc, kind, maps, M, N, K, ep, grp, width, lo);
+  return launch_ar<BN, 128>(lc, kind, maps, M, N, K, ep, grp, width, lo);
 }
 }  // namespace
 
@@ -530,11 +545,13 @@ int gemm_tile_n(const LaunchCtx& lc, const GemmMaps& maps, int M, int N) {
 cudaError_t prepare_gemm_kernels() {
   cudaError_t e = prepare_gemm_t<bf16>();
   if (e == cudaSuccess) e = prepare_gemm_t<f16>();
+  if (e == cudaSuccess) e = set_smem_lo<EPI_SWIGLU>();
+  if (e == cudaSuccess) e = set_smem_lo<EPI_LOGITS>();
   return e;
 }
 
 cudaError_t launch_gemm_tc(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K,
-                           const EpiArgs& ep, int tile_n, const GemmGroup* group) {
+                           const EpiArgs& ep, int tile_n, const GemmGroup* group, bool lo) {
   if (M < 1 || N < 1 || K < BK || (K % BK)) return cudaErrorInvalidValue;
   const GemmGroup grp = group ? *group : GemmGroup{};
   if (grp.mb_expert && (!grp.n_mblocks || (M % BM))) return cudaErrorInvalidValue;
@@ -543,11 +560,13 @@ cudaError_t launch_gemm_tc(const LaunchCtx& lc, int kind, const GemmMaps& maps, 
   // rows: the small-M stage layouts
   const bool dec = !grp.mb_expert && kind != EPI_ROWSCALE;
   const int arows = (dec && M <= 16 && maps.has16) ? 16 : ((dec && M <= 64 && maps.has64) ? 64 : 128);
+  if (lo && !(lc.f16 && maps.has_lo && arows < BM && (kind == EPI_SWIGLU || kind == EPI_LOGITS)))
+    return cudaErrorInvalidValue;
   const bool mid = maps.mid && arows == 128 && !grp.mb_expert;
   if (tile_n != 256 && tile_n != 128 && !(mid && (tile_n == 192 || tile_n == 224))) return cudaErrorInvalidValue;
   if (tile_n == 128) {
     if (!maps.n128) return cudaErrorInvalidValue;
-    return launch_bn<128>(lc, kind, maps, M, N, K, ep, grp, arows, 128);
+    return launch_bn<128>(lc, kind, maps, M, N, K, ep, grp, arows, 128, lo);
   }
-  return launch_bn<256>(lc, kind, maps, M, N, K, ep, grp, arows, tile_n);
+  return launch_bn<256>(lc, kind, maps, M, N, K, ep, grp, arows, tile_n, lo);
 }

@@ -209,7 +209,8 @@ struct GemmMaps {
   CUtensorMap a_lo64;
   bool has16 = false;
   bool has64 = false;
-  bool split = false;
+  bool split = false;   // the operand always has two terms (QKV, fp16 mode)
+  bool has_lo = false;  // a_lo16 and a_lo64 exist
   bool mid = false;
   const GemmMaps* n128 = nullptr;  // the same operands with 128-row weight boxes (128-wide tiles), or null
 };
@@ -234,9 +235,10 @@ struct GemmGroup {
   const int* row_valid = nullptr;
 };
 // tile_n: 256, 224, 192 or 128 (from gemm_tile_n); the residual epilogue writes two
-// norm partials per row and tile, i.e. 2 * ceil(N / tile_n) of them.
+// norm partials per row and tile, i.e. 2 * ceil(N / tile_n) of them. lo: gate/up and
+// logits of at most 64 rows take the operand's second term too (fp16 mode, has_lo).
 cudaError_t launch_gemm_tc(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
-                           int tile_n = 256, const GemmGroup* group = nullptr);
+                           int tile_n = 256, const GemmGroup* group = nullptr, bool lo = false);
 int gemm_tile_n(const LaunchCtx& lc, const GemmMaps& maps, int M, int N);
 
 // ---- projections of few tokens (k_skinny.cu): weights as the 128-row MMA
