@@ -517,6 +517,7 @@ struct Proj {
   LaunchCtx lc;
   bool decode = false;  // o_lo / u_lo were written by this step's producers
   bool tc = false;      // the pass runs on the tcgen05 kernels
+  bool skinny = false;  // the last product ran on launch_skinny
   cudaError_t rc = cudaSuccess;
   // act: activation rows (row stride act_stride elements), M rows. Returns
   // the norm state a RESID producer leaves behind.
@@ -524,6 +525,7 @@ struct Proj {
                 int M, EpiArgs& ep) {
     ep.M = M;
     ep.N = N;
+    skinny = false;
     NormState ns;
     // fp16 mode: the second term of the operand, where its producer left one
     const void* lo = nullptr;
@@ -563,6 +565,7 @@ struct Proj {
       const SkinnyPlan pl = am ? skinny_plan(lc, M, N, K, two) : SkinnyPlan{};
       if (pl.ks > 0) {
         rc = launch_skinny(lc, kind, maps->n128->w, *am, M, N, K, ep, pl);
+        skinny = true;
         ns.parts = (N + 127) / 128;
         return ns;
       }
@@ -809,6 +812,14 @@ int enqueue_prefill(axon_model* m, const int32_t* ids, int B, int S, const int32
     row.rowmap = rowmap;
     CK_RC(enqueue_mlp(m, l, pj, lc, pf, row, M, false, ns));
   }
+  // The LM head's GEMV keeps its loads in flight in L1. Behind the few-token
+  // kernel, which lets its successor start early, it would run from end to end on the
+  // little L1 that kernel's carveout left: there it waits for the SMs to drain (prompt of 2
+  // tokens, whole vocabulary, fp16: 8B width, 2 layers, 448 -> 348 us, 32B width, 1 layer, 684 ->
+  // 440; of 16 at 0.5B width, 2 layers, 198 -> 144; a batch of 4 decode tokens and a short chunk, bf16,
+  // 8B width 453 -> 359). The prefill GEMM lets nothing start early.
+  LaunchCtx head_lc = lc;
+  if (pj.skinny && m->layers[m->L - 1].Fl) head_lc.pdl = false;
   EpiArgs h = base_epi(m);
   h.S = S;
   h.rowmap = rowmap;
@@ -843,7 +854,7 @@ int enqueue_prefill(axon_model* m, const int32_t* ids, int B, int S, const int32
         CK(launch_skinny(lc, EPI_LOGITS, m->v_head, m->am_last, nb, m->V, D, hg, pl, b0));
         continue;
       }
-      CK(launch_gemv(lc, EPI_LOGITS, m->fp32, m->head, m->V, D, static_cast<char*>(m->a_last) + off, D, nb, hg,
+      CK(launch_gemv(head_lc, EPI_LOGITS, m->fp32, m->head, m->V, D, static_cast<char*>(m->a_last) + off, D, nb, hg,
                      m->splitk, m->a_lo_last ? static_cast<char*>(m->a_lo_last) + off : nullptr));
     }
     CK(launch_finalize_varlen(lc, m->keys, B, vl->cu, 0, B, next, vl->ctx));
@@ -863,7 +874,7 @@ int enqueue_prefill(axon_model* m, const int32_t* ids, int B, int S, const int32
     h.M = B;
     h.N = m->V;
     pbeg(pf, "prefill_lm_head");
-    CK(launch_gemv(lc, EPI_LOGITS, m->fp32, m->head, m->V, D, static_cast<char*>(m->a) + off,
+    CK(launch_gemv(head_lc, EPI_LOGITS, m->fp32, m->head, m->V, D, static_cast<char*>(m->a) + off,
                    static_cast<long long>(S) * D, B, h, m->splitk,
                    m->a_lo ? static_cast<char*>(m->a_lo) + off : nullptr));
     pend(pf, whd + B * (D * es + (logits ? 4.0 * m->V : 0.0)), 2.0 * B * m->V * D);
