@@ -729,16 +729,17 @@ struct VarlenBatch {
 // Whether a prefill's attention runs on the tcgen05 kernel (k_attn_tc.cu) or
 // on the mma.sync one. A tcgen05 CTA takes about 2 us longer to its first
 // output and holds a whole SM, so that the next kernels' CTAs cannot start
-// early beside it; it wins where key steps or waves amortise that. Whole
-// passes, mma.sync / tcgen05: 8B width 2 layers S = 256 418 / 424 us, 384 479 /
-// 477, 512 521 / 509; B = 16 S = 128 1365 / 1355, S = 256 2644 / 2606; 0.5B
-// width 4 layers S = 384 366 / 370, 512 380 / 378, B = 16 S = 256 853 / 841.
-// Variable-length batches may hold long contexts behind short chunks (8B width,
-// 30 contexts of up to 600 tokens and a 64-token chunk: 451 / 438) and take it
+// early beside it; it wins where key steps or waves amortise that, at head_dim 64 (half
+// the work per key step) later. Whole passes in bf16, mma.sync / tcgen05: 8B width, 2 layers, S =
+// 256 364 / 364 us, 384 440 / 434, 512 480 / 467; B = 8 S = 256 1329 / 1314; 16B mixture of
+// experts, 2 layers, S = 384 459 / 450; 0.5B width, 4 layers, S = 448 270 / 278, 512 278 / 281, 640
+// 310 / 308, 1024 388 / 368, B = 16 S = 256 600 / 594; 135M width, 6 layers, S = 512 318 / 323, 640
+// 335 / 338, 768 352 / 348. Variable-length batches may hold long contexts behind short chunks (8B
+// width, 30 contexts of up to 600 tokens and a 64-token chunk: 451 / 438) and take it
 // unless they have GEMV-sized projections (at most 64 rows).
-bool attn_on_tcgen05(int M, int S, bool varlen) {
+bool attn_on_tcgen05(int M, int S, int d, bool varlen) {
   if (varlen) return M > 64;
-  return S > 384 || (S >= 256 && M >= 2048);
+  return S > (d == 128 ? 384 : 576) || (S >= 256 && M >= 2048);
 }
 
 int enqueue_prefill(axon_model* m, const int32_t* ids, int B, int S, const int32_t* bt, int logits_mode, float* logits,
@@ -755,7 +756,7 @@ int enqueue_prefill(axon_model* m, const int32_t* ids, int B, int S, const int32
   Proj pj{m, lc};
   pj.tc = tc;
   const int D = m->D, Hd = m->H * m->d;
-  const bool attn_tc = !m->fp32 && attn_on_tcgen05(M, S, vl != nullptr);
+  const bool attn_tc = !m->fp32 && attn_on_tcgen05(M, S, m->d, vl != nullptr);
   pbeg(pf, "embed");
   CK(launch_embed(lc, m->fp32, m->embed, m->V, D, ids, M, m->x, m->a, m->L > 0 ? m->layers[0].g1 : m->gf, m->ss,
                   m->Pmax, m->rinv, m->cfg.rms_norm_eps, m->err, m->a_lo));
