@@ -339,12 +339,15 @@ AXON_DEV void attn_decode_item(const AttnArgs& p, int s, int g, int b, uint8_t* 
   if constexpr (LL::on) {
     ll.template load_q<HD>(qa, (static_cast<long long>(b) * p.H + g * HPG + r) * HD, r < HPG, q);
   } else {
-  const uint16_t* qg1 = paired ? static_cast<const uint16_t*>(p.q_lo) + qoff + r * HD : qg + (r + 8) * HD;
-  load_q<HD>(qa, r < HPG ? qg + r * HD : nullptr, (paired ? r : r + 8) < HPG ? qg1 : nullptr, q);
+    const uint16_t* qg1 = paired ? static_cast<const uint16_t*>(p.q_lo) + qoff + r * HD : qg + (r + 8) * HD;
+    load_q<HD>(qa, r < HPG ? qg + r * HD : nullptr, (paired ? r : r + 8) < HPG ? qg1 : nullptr, q);
   }
   // LL: the newest token's key and value have not reached the cache; they
-  // replace their row of the staged block
-  const int jnew = LL::on && p.ctx[b] + 1 == T ? (T - 1) >> 4 : -1;
+  // replace their row of the staged block. They are awaited for a position outside
+  // the cache (reported) too: their words may not be written for the next layer
+  // before their readers are done with this one.
+  const int jnew = LL::on ? (T - 1) >> 4 : -1;
+  const bool fresh = LL::on && p.ctx[b] + 1 == T;
 
   WarpState<HD> st;
   st.init();
@@ -362,7 +365,8 @@ AXON_DEV void attn_decode_item(const AttnArgs& p, int s, int g, int b, uint8_t* 
       __syncwarp();
       if constexpr (LL::on) {
         if (j == jnew) {
-          ll.template patch<HD>(wbase + stg * 2 * TILE, (static_cast<long long>(b) * p.G + g) * HD, (T - 1) & 15, lane);
+          ll.template patch<HD>(wbase + stg * 2 * TILE, (static_cast<long long>(b) * p.G + g) * HD, (T - 1) & 15, lane,
+                                fresh);
           __syncwarp();
         }
       }

@@ -27,7 +27,8 @@
 // two terms of one value; fp32 for the residual and the norm partials.
 //   Reuse: each buffer has one writing phase per layer, and a phase cannot begin
 // writing layer l + 1 before every reader of layer l is done: its inputs depend,
-// through the phases between, on the outputs of all of that buffer's readers.
+// through the phases between, on the outputs of all of that buffer's readers (the
+// newest k and v are awaited even where their position lies outside the cache).
 //   Flags: epoch + layer + 1, the epoch advanced by L + 1 with every launch, so that
 // what an earlier layer or launch left never matches.
 // The first layer's operand is the embedding, which every CTA computes itself.
@@ -171,9 +172,10 @@ struct LLAttn {
       }
     }
   }
-  // The newest token's key and value into row `tok` of a staged block [K | V].
+  // The newest token's key and value, into row `tok` of a staged block [K | V] if
+  // that is their place.
   template <int HD>
-  AXON_DEV void patch(uint32_t stage, long long off, int tok, int lane) const {
+  AXON_DEV void patch(uint32_t stage, long long off, int tok, int lane, bool store) const {
     constexpr int VECS = HD / 4;  // four values per vector
     constexpr int N = 2 * VECS / 32;
     uint4 w[N];
@@ -182,6 +184,7 @@ struct LLAttn {
       return (kv ? v : k) + static_cast<int>(off >> 2) + (t - kv * VECS);
     };
     poll_vecs<N>(w, src, flag, g, s_abort, err);
+    if (!store) return;
 #pragma unroll
     for (int u = 0; u < N; ++u) {
       const int t = lane + u * 32, kv = t / VECS, i = t - kv * VECS;

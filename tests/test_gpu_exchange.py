@@ -76,3 +76,26 @@ def test_batch_sizes_in_turn(prec):
         assert ax.axon_check_device(m)[0] == 0
     finally:
         ax.axon_free(m)
+
+
+@pytest.mark.parametrize("prec", ["bf16", "fp16"])
+def test_position_outside_the_cache_is_reported_and_nothing_else(prec):
+    """A sequence whose cache is full: DEVERR_POS (4) and no wait that ran out (8),
+    while the other sequences of the step are as without it."""
+    ax = _ax()
+    shape = dict(PIECES, F=192, L=6)
+    w = gpu_weights(shape)
+    m = create(shape, w, max_batch=3, max_context=32, fp16=prec == "fp16")
+    try:
+        ids = si.make_ids(3, 9, shape["V"], seed=5)
+        _, nxt = run_prefill(m, ids, ax.AXON_LOGITS_LAST, shape["V"])
+        ref, _ = decode_steps(m, nxt, [9] * 3, 1, shape["V"])
+        for full in (32, 40):
+            tok, ctx = torch.from_numpy(nxt).cuda(), torch.tensor([9, full, 9], dtype=torch.int32, device="cuda")
+            logits = torch.empty(3, shape["V"], device="cuda")
+            ax.axon_decode_step(m, tok, ctx, logits=logits, next_tokens=torch.empty_like(tok))
+            assert ax.axon_check_device(m)[1] == 4
+            assert np.array_equal(logits.cpu().numpy()[[0, 2]], ref[[0, 2], 0])
+            assert ctx.tolist() == [10, full + 1, 10]
+    finally:
+        ax.axon_free(m)
