@@ -940,6 +940,7 @@ PersistArgs persist_args(const axon_model* m, const int32_t* tokens, int B, int3
     *ll[i] = at;
     at += persist_ll_vecs(m, i);
   }
+  a.ll_vecs = static_cast<unsigned>(at - m->persist_ll);
   a.keys = m->keys;
   a.attn_part = attn_part;
   a.attn_cnt = attn_cnt;
@@ -1856,6 +1857,15 @@ void axon_free(axon_model* m) {
   if (!m) return;
   cudaDeviceSynchronize();
   free_model(m);
+}
+
+// Not in the header: where the flags of the persistent step's exchange stand (tests
+// of their wrap). Between steps only.
+int axon_internal_persist_epoch(axon_model* m, uint32_t epoch) {
+  if (!m || !m->pgrid) return AXON_ERR_INVALID_ARG;
+  CK(cudaDeviceSynchronize());
+  CK(cudaMemcpy(&m->pgrid->epoch, &epoch, sizeof(epoch), cudaMemcpyHostToDevice));
+  return AXON_OK;
 }
 
 }  // extern "C"

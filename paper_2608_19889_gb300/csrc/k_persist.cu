@@ -30,7 +30,9 @@
 // through the phases between, on the outputs of all of that buffer's readers (the
 // newest k and v are awaited even where their position lies outside the cache).
 //   Flags: epoch + layer + 1, the epoch advanced by L + 1 with every launch, so that
-// what an earlier layer or launch left never matches.
+// what an earlier layer or launch left never matches. Before the 32-bit flags would
+// wrap (after some 10^8 steps) the last CTA of a launch clears the buffers and starts the
+// epoch anew; 0 is never a flag.
 // The first layer's operand is the embedding, which every CTA computes itself.
 //
 // Work split: a projection phase is cut into items of 16 weight rows x all
@@ -364,7 +366,7 @@ struct PhaseIO {
 //
 // Per item the consumer warps only run the products and the cross-warp sum;
 // the item's 16 x B sums go to a shared buffer and the epilogues run in
-// batches of up to 64 items, eight lanes per (item, token), so that their
+// batches of up to 32 / B items, eight lanes per (item, token), so that their
 // global reads overlap instead of stalling the weight stream item after item;
 // the first batch's reads are requested before the products. The LM head's
 // argmax keeps a per-CTA best key per token in shared memory and commits it
@@ -837,9 +839,15 @@ __global__ void __launch_bounds__(PTHREADS, 1) persist_decode_kernel(PersistArgs
       if (A.next) A.next[b] = static_cast<int>(0xffffffffu - static_cast<uint32_t>(k & 0xffffffffull));
       A.ctx[b] += 1;
     }
+    uint32_t next = epoch + static_cast<uint32_t>(A.L) + 1u;
+    if (next > 0xfffffffeu - static_cast<uint32_t>(A.L)) {  // its last flag would be next + L + 1
+#pragma unroll 1
+      for (unsigned i = 0; i < A.ll_vecs; ++i) A.ll_ao[i] = make_uint4(0u, 0u, 0u, 0u);
+      next = 0u;
+    }
     g->abort = 0u;
     g->exit = 0u;
-    g->epoch = epoch + static_cast<uint32_t>(A.L) + 1u;
+    g->epoch = next;
   }
 }
 

@@ -318,7 +318,9 @@ struct PersistArgs {
   const float2* rope;
   // Exchange buffers of flagged 8-byte words (k_persist.cu): operand with norm
   // partials, and residual, after the O (..o) and the down projection (..d), q, the
-  // newest k and v, attention and SwiGLU outputs.
+  // newest k and v, attention and SwiGLU outputs; one allocation of ll_vecs vectors
+  // from ll_ao on.
+  unsigned ll_vecs;
   uint4* ll_ao;
   uint4* ll_ad;
   uint4* ll_xo;

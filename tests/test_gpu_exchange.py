@@ -3,6 +3,8 @@ operands that stage in several pieces (an MLP wide enough at head_dim 64), steps
 of different batch sizes in turn on one model (what an earlier, larger batch left
 in the buffers must not be taken for this step's), and several layers and steps
 (flags of earlier layers and launches)."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -99,3 +101,33 @@ def test_position_outside_the_cache_is_reported_and_nothing_else(prec):
             assert ctx.tolist() == [10, full + 1, 10]
     finally:
         ax.axon_free(m)
+
+
+def test_flags_start_anew_before_they_wrap():
+    """Steps on both sides of the 32-bit wrap, the ones after it with more sequences than
+    any before (words that nothing has written yet): bit-identical to a model whose
+    flags are far from it."""
+    ax = _ax()
+    shape = dict(PIECES, F=192)
+    w = gpu_weights(shape)
+    ids = si.make_ids(8, 9, shape["V"], seed=5)
+    runs = []
+    for epoch in (None, 2**32 - 9):  # steps of L + 1 = 4 flags: two fit
+        m = create(shape, w, max_batch=8, max_context=32)
+        try:
+            _, nxt = run_prefill(m, ids, ax.AXON_LOGITS_LAST, shape["V"])
+            if epoch is not None:
+                assert ax.lib().axon_internal_persist_epoch(m, ctypes.c_uint32(epoch)) == 0
+            out, lens = [], np.full(8, 9, dtype=np.int32)
+            for n in (2, 1, 8, 3, 8):
+                tok, ctx = torch.from_numpy(nxt[:n].copy()).cuda(), torch.from_numpy(lens[:n].copy()).cuda()
+                logits = torch.empty(n, shape["V"], device="cuda")
+                ax.axon_decode_step(m, tok, ctx, logits=logits, next_tokens=torch.empty_like(tok))
+                out.append(logits.cpu().numpy())
+                lens[:n] += 1
+            assert ax.axon_check_device(m)[0] == 0
+            runs.append(out)
+        finally:
+            ax.axon_free(m)
+    for a, b in zip(*runs):
+        assert np.array_equal(a, b)
