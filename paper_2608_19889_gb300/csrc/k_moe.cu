@@ -40,7 +40,9 @@ constexpr int FUSED_GATHER_MAX = 32;
 
 // Token t: softmax of its router logits, top-k by repeated arg-max over
 // (probability, lowest index), the weights (renormalised over the k chosen
-// when norm_topk). One warp; lg is the warp's [E] scratch.
+// when norm_topk). One warp; lg is the warp's [E] scratch. An expert whose
+// probability is not a number ranks below all others, so that k valid experts are
+// chosen whatever the logits; their weights are then not numbers either.
 AXON_DEV void route_token(const MoeArgs& a, int t, float* lg, int lane) {
   const int E = a.E, k = a.k;
   __syncwarp();
@@ -52,7 +54,7 @@ AXON_DEV void route_token(const MoeArgs& a, int t, float* lg, int lane) {
   float den = 0.f;
   for (int e = lane; e < E; e += 32) {
     const float p = expf(lg[e] - mx);
-    lg[e] = p;
+    lg[e] = p == p ? p : -1.f;
     den += p;
   }
   den = warp_sum(den);
@@ -60,7 +62,7 @@ AXON_DEV void route_token(const MoeArgs& a, int t, float* lg, int lane) {
   float wsum = 0.f, wk[8];
   int ik[8];
   for (int j = 0; j < k; ++j) {
-    float bv = -1.f;
+    float bv = -1.5f;  // above the experts taken
     int bi = 0x7fffffff;
     for (int e = lane; e < E; e += 32) {
       const float p = lg[e];

@@ -42,3 +42,27 @@ def test_rows_at_the_edges_of_the_routing_launches(rows, prec):
         check(lg, ref, tol=tiny_tol(prec), what=f"{rows} rows ({prec})")
     finally:
         ax.axon_free(m)
+
+
+@pytest.mark.parametrize("S", [3, 20, 150])
+def test_token_whose_router_logits_are_not_numbers(S):
+    """It is routed to valid, distinct experts, and the other sequence is as without it."""
+    ax = _ax()
+    shape = MOE2
+    w = gpu_weights(shape)
+    ids = si.make_ids(2, S, shape["V"] - 1, seed=S)
+    w["model.embed_tokens.weight"][shape["V"] - 1] = float("nan")
+    m = create(shape, w, max_batch=2, max_context=160, max_prefill_tokens=2 * S)
+    try:
+        rec = torch.full((shape["L"], 2 * S, shape["top_k"]), -1, dtype=torch.int32, device="cuda")
+        ref, _ = run_prefill(m, ids, ax.AXON_LOGITS_LAST, shape["V"])
+        ids[0, -1] = shape["V"] - 1
+        ax.axon_moe_routing_record(m, rec, 2 * S)
+        lg, _ = run_prefill(m, ids, ax.AXON_LOGITS_LAST, shape["V"])
+        assert ax.axon_check_device(m)[0] == 0
+        for l in _moe_layers(shape):
+            for row in rec[l].tolist():
+                assert len(set(row)) == shape["top_k"] and 0 <= min(row) and max(row) < shape["n_experts"]
+        assert (lg[0] != lg[0]).all() and (lg[1] == ref[1]).all()
+    finally:
+        ax.axon_free(m)
