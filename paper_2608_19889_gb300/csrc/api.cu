@@ -116,8 +116,8 @@ struct axon_model {
   ActMaps am_a{}, am_o{}, am_last{};
   std::map<int, ActMaps> am_u;
   CUtensorMap t_a{}, t_o{}, t_alo{};
-  CUtensorMap t_a16{}, t_o16{}, t_alo16{};  // the same in boxes of 16 rows (decode GEMMs)
-  CUtensorMap t_a64{}, t_o64{}, t_alo64{};  // and of 64 rows
+  CUtensorMap t_a16{}, t_alo16{};  // the same in boxes of 16 rows (few tokens)
+  CUtensorMap t_a64{}, t_alo64{};  // and of 64 rows
   // decode graphs
   cudaStream_t cap_stream = nullptr;
   std::map<GraphKey, cudaGraphExec_t> graphs;
@@ -571,7 +571,7 @@ struct Proj {
       }
     }
     const int tn = gemm_tile_n(lc, *maps, M, N);
-    const bool gemm_lo = lo != nullptr && maps->has_lo && (kind == EPI_SWIGLU || kind == EPI_LOGITS) && M <= (decode ? 8 : 64);
+    const bool gemm_lo = lo != nullptr && maps->has_lo && M <= (decode ? 8 : 64);
     rc = launch_gemm_tc(lc, kind, *maps, M, N, K, ep, tn, nullptr, gemm_lo);
     ns.parts = 2 * ((N + tn - 1) / tn);
     return ns;
@@ -1503,9 +1503,7 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
       ok = make_tma_2d_16(&m->t_asorted, m->moe_a_sorted, m->R_cap, D, 128, m->f16) &&
            make_tma_2d_16(&m->t_usorted, m->moe_u_sorted, m->R_cap, m->Fe, 128, m->f16);
     if (ok && m->a_lo) ok = make_tma_2d_16(&m->t_alo, m->a_lo, Mcap, D, 128, m->f16);
-    ok = ok && make_tma_2d_16(&m->t_a16, m->a, Mcap, D, 16, m->f16) &&
-         make_tma_2d_16(&m->t_o16, m->o, Mcap, Hd, 16, m->f16) &&
-         make_tma_2d_16(&m->t_a64, m->a, Mcap, D, 64, m->f16) && make_tma_2d_16(&m->t_o64, m->o, Mcap, Hd, 64, m->f16);
+    ok = ok && make_tma_2d_16(&m->t_a16, m->a, Mcap, D, 16, m->f16) && make_tma_2d_16(&m->t_a64, m->a, Mcap, D, 64, m->f16);
     if (ok && m->a_lo)
       ok = make_tma_2d_16(&m->t_alo16, m->a_lo, Mcap, D, 16, m->f16) &&
            make_tma_2d_16(&m->t_alo64, m->a_lo, Mcap, D, 64, m->f16);
@@ -1515,16 +1513,15 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
     for (const LayerW& w : m->layers)
       if (w.Fl && !m->am_u.count(w.Fl))
         ok = ok && make_act_maps(&m->am_u[w.Fl], m->u, m->u_lo, Mcap, m->cfg.max_batch, w.Fl, m->f16);
-    // lo: the operand is `a`, which has a second term in fp16 mode
-    auto small_a = [&](GemmMaps& g, const CUtensorMap& a16, const CUtensorMap& a64, bool lo) {
-      g.a16 = a16;
-      g.a64 = a64;
-      if (lo && m->a_lo) {
+    auto small_a = [&](GemmMaps& g) {
+      g.a16 = m->t_a16;
+      g.a64 = m->t_a64;
+      g.few = true;
+      if (m->a_lo) {
         g.a_lo16 = m->t_alo16;
         g.a_lo64 = m->t_alo64;
         g.has_lo = true;
       }
-      g.has16 = g.has64 = true;
     };
     for (int l = 0; l < m->L && ok; ++l) {
       LayerW& w = m->layers[l];
@@ -1536,19 +1533,13 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
       }
       w.m_o.a = m->t_o;
       ok = ok && make_tma_2d_16(&w.m_o.w, w.wo, D, Hd, 256, m->f16);
-      small_a(w.m_qkv, m->t_a16, m->t_a64, true);
-      small_a(w.m_o, m->t_o16, m->t_o64, false);
       if (w.Fl) {
         w.m_gu.a = m->t_a;
         ok = ok && make_tma_2d_16(&w.m_gu.w, w.wgu, 2 * w.Fl, D, 256, m->f16);
         // the down projection reads u with this layer's row stride
         ok = ok && make_tma_2d_16(&w.m_d.a, m->u, Mcap, w.Fl, 128, m->f16);
         ok = ok && make_tma_2d_16(&w.m_d.w, w.wd, D, w.Fl, 256, m->f16);
-        small_a(w.m_gu, m->t_a16, m->t_a64, true);
-        CUtensorMap u16, u64;
-        ok = ok && make_tma_2d_16(&u16, m->u, Mcap, w.Fl, 16, m->f16) &&
-             make_tma_2d_16(&u64, m->u, Mcap, w.Fl, 64, m->f16);
-        small_a(w.m_d, u16, u64, false);
+        small_a(w.m_gu);
       }
       if (w.moe) {
         const int E = m->E, Fe = m->Fe;
@@ -1575,7 +1566,7 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
     }
     m->m_head.a = m->t_a;
     ok = ok && make_tma_2d_16(&m->m_head.w, m->head, V, D, 256, m->f16);
-    small_a(m->m_head, m->t_a16, m->t_a64, true);
+    small_a(m->m_head);
     auto mid_w = [&](GemmMaps& g, const void* w, int N, int K) {
       ok = ok && make_tma_2d_16(&g.w192, w, N, K, 192, m->f16) && make_tma_2d_16(&g.w224, w, N, K, 224, m->f16);
       g.mid = true;
@@ -1590,7 +1581,7 @@ int axon_model_create(const axon_config* cfg, const axon_tensor* weights, int32_
       }
     }
     mid_w(m->m_head, m->head, V, D);
-    // decode projections: weight boxes of 128 rows, activation boxes of 8..64 token rows
+    // weight boxes of 128 rows: the few-token kernel's, and the GEMM's 128-wide tiles
     for (int l = 0; l < m->L && ok; ++l) {
       LayerW& w = m->layers[l];
       ok = make_tma_2d_16(&w.v_qkv, w.wqkv, m->Nqkv, D, 128, m->f16) && make_tma_2d_16(&w.v_o, w.wo, D, Hd, 128, m->f16);

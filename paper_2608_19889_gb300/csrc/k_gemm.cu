@@ -27,8 +27,6 @@
 
 #include <cudaTypedefs.h>
 
-#include <type_traits>
-
 namespace {
 
 constexpr int BM = 128, BK = 64, GROUP_M = 8;
@@ -42,13 +40,13 @@ constexpr int NUM_THREADS = 64 + 32 * EPI_WARPS;
 // accumulator. The ring takes as many stages as fit in 200 KB, at most 6
 // (BN 256: 4, split 3; BN 128: 6, split 4).
 //
-// AROWS < 128 (at most AROWS activation rows, decode: 16 or 64): each stage
+// AROWS < 128 (gate/up and logits of at most AROWS activation rows, 16 or 64, whose
+// weights are too wide for the few-token kernel): each stage
 // holds [A (AROWS rows) | A_lo (AROWS rows, SPLIT) | B]; the MMA still reads
 // 128 A rows from the tile, rows AROWS..127 falling in the same stage's
 // following bytes (landed, so stable; their accumulator rows are never
 // stored). Without the padding rows a stage is smaller, so more of them --
 // more weight bytes in flight per SM -- fit (up to 12).
-//
 //
 // RING: the ring's byte budget (the residual kind's epilogue staging takes 32 KB).
 template <bool SPLIT, int BN_, int AROWS = 128, int RING = 200 * 1024>
@@ -461,21 +459,15 @@ template <int KIND, typename T16, bool SPLIT>
 cudaError_t set_smem() {
   cudaError_t e = set_smem1<KIND, T16, SPLIT, 256, 128>();
   if (e == cudaSuccess) e = set_smem1<KIND, T16, SPLIT, 128, 128>();
-  if constexpr (KIND != EPI_ROWSCALE) {  // the small-M layouts (decode kinds)
-    if (e == cudaSuccess) e = set_smem1<KIND, T16, SPLIT, 256, 16>();
-    if (e == cudaSuccess) e = set_smem1<KIND, T16, SPLIT, 128, 16>();
-    if (e == cudaSuccess) e = set_smem1<KIND, T16, SPLIT, 256, 64>();
-    if (e == cudaSuccess) e = set_smem1<KIND, T16, SPLIT, 128, 64>();
-  }
   return e;
 }
-// The small-M layouts of a two-term operand (fp16 mode), beside QKV's.
-template <int KIND>
-cudaError_t set_smem_lo() {
-  cudaError_t e = set_smem1<KIND, f16, true, 256, 16>();
-  if (e == cudaSuccess) e = set_smem1<KIND, f16, true, 128, 16>();
-  if (e == cudaSuccess) e = set_smem1<KIND, f16, true, 256, 64>();
-  if (e == cudaSuccess) e = set_smem1<KIND, f16, true, 128, 64>();
+// The small-M layouts.
+template <int KIND, typename T16, bool SPLIT>
+cudaError_t set_smem_few() {
+  cudaError_t e = set_smem1<KIND, T16, SPLIT, 256, 16>();
+  if (e == cudaSuccess) e = set_smem1<KIND, T16, SPLIT, 128, 16>();
+  if (e == cudaSuccess) e = set_smem1<KIND, T16, SPLIT, 256, 64>();
+  if (e == cudaSuccess) e = set_smem1<KIND, T16, SPLIT, 128, 64>();
   return e;
 }
 template <typename T16>
@@ -486,37 +478,43 @@ cudaError_t prepare_gemm_t() {
   if (e == cudaSuccess) e = set_smem<EPI_SWIGLU, T16, false>();
   if (e == cudaSuccess) e = set_smem<EPI_LOGITS, T16, false>();
   if (e == cudaSuccess) e = set_smem<EPI_ROWSCALE, T16, false>();
+  if (e == cudaSuccess) e = set_smem_few<EPI_SWIGLU, T16, false>();
+  if (e == cudaSuccess) e = set_smem_few<EPI_LOGITS, T16, false>();
   return e;
 }
-template <typename T16, int BN, int AROWS>
+template <typename T16, int BN>
 cudaError_t launch_t(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
-                     const GemmGroup& grp, int width, bool lo) {
-  if constexpr (AROWS < BM && std::is_same<T16, f16>::value) {
-    if (lo && kind == EPI_SWIGLU) return launch_kind<EPI_SWIGLU, T16, true, BN, AROWS>(lc, maps, M, N, K, ep, grp, width);
-    if (lo && kind == EPI_LOGITS) return launch_kind<EPI_LOGITS, T16, true, BN, AROWS>(lc, maps, M, N, K, ep, grp, width);
-  }
+                     const GemmGroup& grp, int width) {
   switch (kind) {
     case EPI_QKV:
-      return maps.split ? launch_kind<EPI_QKV, T16, true, BN, AROWS>(lc, maps, M, N, K, ep, grp, width)
-                        : launch_kind<EPI_QKV, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, grp, width);
-    case EPI_RESID: return launch_kind<EPI_RESID, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, grp, width);
-    case EPI_SWIGLU: return launch_kind<EPI_SWIGLU, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, grp, width);
+      return maps.split ? launch_kind<EPI_QKV, T16, true, BN, 128>(lc, maps, M, N, K, ep, grp, width)
+                        : launch_kind<EPI_QKV, T16, false, BN, 128>(lc, maps, M, N, K, ep, grp, width);
+    case EPI_RESID: return launch_kind<EPI_RESID, T16, false, BN, 128>(lc, maps, M, N, K, ep, grp, width);
+    case EPI_SWIGLU: return launch_kind<EPI_SWIGLU, T16, false, BN, 128>(lc, maps, M, N, K, ep, grp, width);
     case EPI_ROWSCALE: return launch_kind<EPI_ROWSCALE, T16, false, BN, 128>(lc, maps, M, N, K, ep, grp, width);
-    default: return launch_kind<EPI_LOGITS, T16, false, BN, AROWS>(lc, maps, M, N, K, ep, grp, width);
+    default: return launch_kind<EPI_LOGITS, T16, false, BN, 128>(lc, maps, M, N, K, ep, grp, width);
   }
 }
+// The small-M layouts (gate/up and logits); LO: a two-term operand.
+template <typename T16, bool LO, int BN, int AROWS>
+cudaError_t launch_few(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep) {
+  return kind == EPI_SWIGLU ? launch_kind<EPI_SWIGLU, T16, LO, BN, AROWS>(lc, maps, M, N, K, ep, GemmGroup{}, BN)
+                            : launch_kind<EPI_LOGITS, T16, LO, BN, AROWS>(lc, maps, M, N, K, ep, GemmGroup{}, BN);
+}
 template <int BN, int AROWS>
-cudaError_t launch_ar(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
-                      const GemmGroup& grp, int width, bool lo) {
-  return lc.f16 ? launch_t<f16, BN, AROWS>(lc, kind, maps, M, N, K, ep, grp, width, lo)
-                : launch_t<bf16, BN, AROWS>(lc, kind, maps, M, N, K, ep, grp, width, lo);
+cudaError_t launch_few_t(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
+                         bool lo) {
+  if (!lc.f16) return launch_few<bf16, false, BN, AROWS>(lc, kind, maps, M, N, K, ep);
+  return lo ? launch_few<f16, true, BN, AROWS>(lc, kind, maps, M, N, K, ep)
+            : launch_few<f16, false, BN, AROWS>(lc, kind, maps, M, N, K, ep);
 }
 template <int BN>
 cudaError_t launch_bn(const LaunchCtx& lc, int kind, const GemmMaps& maps, int M, int N, int K, const EpiArgs& ep,
                       const GemmGroup& grp, int arows, int width, bool lo) {
-  if (arows == 16) return launch_ar<BN, 16>(lc, kind, maps, M, N, K, ep, grp, width, lo);
-  if (arows == 64) return launch_ar<BN, 64>(lc, kind, maps, M, N, K, ep, grp, width, lo);
-  return launch_ar<BN, 128>(lc, kind, maps, M, N, K, ep, grp, width, lo);
+  if (arows == 16) return launch_few_t<BN, 16>(lc, kind, maps, M, N, K, ep, lo);
+  if (arows == 64) return launch_few_t<BN, 64>(lc, kind, maps, M, N, K, ep, lo);
+  return lc.f16 ? launch_t<f16, BN>(lc, kind, maps, M, N, K, ep, grp, width)
+                : launch_t<bf16, BN>(lc, kind, maps, M, N, K, ep, grp, width);
 }
 }  // namespace
 
@@ -545,8 +543,8 @@ int gemm_tile_n(const LaunchCtx& lc, const GemmMaps& maps, int M, int N) {
 cudaError_t prepare_gemm_kernels() {
   cudaError_t e = prepare_gemm_t<bf16>();
   if (e == cudaSuccess) e = prepare_gemm_t<f16>();
-  if (e == cudaSuccess) e = set_smem_lo<EPI_SWIGLU>();
-  if (e == cudaSuccess) e = set_smem_lo<EPI_LOGITS>();
+  if (e == cudaSuccess) e = set_smem_few<EPI_SWIGLU, f16, true>();
+  if (e == cudaSuccess) e = set_smem_few<EPI_LOGITS, f16, true>();
   return e;
 }
 
@@ -558,10 +556,9 @@ cudaError_t launch_gemm_tc(const LaunchCtx& lc, int kind, const GemmMaps& maps, 
   if (kind == EPI_ROWSCALE && !grp.mb_expert) return cudaErrorInvalidValue;
   // at most 16 (64) rows -- one M block -- and activation boxes of 16 (64)
   // rows: the small-M stage layouts
-  const bool dec = !grp.mb_expert && kind != EPI_ROWSCALE;
-  const int arows = (dec && M <= 16 && maps.has16) ? 16 : ((dec && M <= 64 && maps.has64) ? 64 : 128);
-  if (lo && !(lc.f16 && maps.has_lo && arows < BM && (kind == EPI_SWIGLU || kind == EPI_LOGITS)))
-    return cudaErrorInvalidValue;
+  const bool few = maps.few && !grp.mb_expert && (kind == EPI_SWIGLU || kind == EPI_LOGITS);
+  const int arows = !few || M > 64 ? 128 : (M <= 16 ? 16 : 64);
+  if (lo && !(lc.f16 && maps.has_lo && arows < BM)) return cudaErrorInvalidValue;
   const bool mid = maps.mid && arows == 128 && !grp.mb_expert;
   if (tile_n != 256 && tile_n != 128 && !(mid && (tile_n == 192 || tile_n == 224))) return cudaErrorInvalidValue;
   if (tile_n == 128) {

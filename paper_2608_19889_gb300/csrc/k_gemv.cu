@@ -1,8 +1,8 @@
 // Decode-side kernels: the weight-streaming projection (skinny GEMV on
 // tensor cores), the embedding gather and the greedy-token finaliser.
 //
-// Projection layout: one CTA owns 16 consecutive weight rows and all B <= 64
-// tokens; its KW warps split K into 64-wide chunks. Each lane streams 2 rows
+// Projection layout: one CTA owns 16 consecutive weight rows and all B <= 16 (logits:
+// 64) tokens; its KW warps split K into 64-wide chunks. Each lane streams 2 rows
 // x 32 bytes per chunk with 16-byte L1-bypassing loads (4 lanes cover 128
 // contiguous bytes of a row), so the whole matrix is read exactly once at
 // full 128-byte-line efficiency. Products run on mma.sync m16n8k16 with the
@@ -345,16 +345,18 @@ template <int NT, typename T16, bool LO>
 cudaError_t gemv_nt_lo(const LaunchCtx& lc, int kind, const T16* w, int N, int K, const T16* a, long long st, int B,
                        const EpiArgs& ep, SplitK sk, const T16* al) {
   const dim3 grid((N + 15) / 16, sk.count), block(GEMV_KW * 32);
-  switch (kind) {
-    case EPI_QKV:
-      return launch_k(lc, gemv_mma_kernel<NT, EPI_QKV, T16, LO>, grid, block, 0, w, N, K, a, st, B, ep, sk, al);
-    case EPI_RESID:
-      return launch_k(lc, gemv_mma_kernel<NT, EPI_RESID, T16, LO>, grid, block, 0, w, N, K, a, st, B, ep, sk, al);
-    case EPI_SWIGLU:
-      return launch_k(lc, gemv_mma_kernel<NT, EPI_SWIGLU, T16, LO>, grid, block, 0, w, N, K, a, st, B, ep, sk, al);
-    default:
-      return launch_k(lc, gemv_mma_kernel<NT, EPI_LOGITS, T16, LO>, grid, block, 0, w, N, K, a, st, B, ep, sk, al);
+  if constexpr (NT <= 2) {
+    switch (kind) {
+      case EPI_QKV:
+        return launch_k(lc, gemv_mma_kernel<NT, EPI_QKV, T16, LO>, grid, block, 0, w, N, K, a, st, B, ep, sk, al);
+      case EPI_RESID:
+        return launch_k(lc, gemv_mma_kernel<NT, EPI_RESID, T16, LO>, grid, block, 0, w, N, K, a, st, B, ep, sk, al);
+      case EPI_SWIGLU:
+        return launch_k(lc, gemv_mma_kernel<NT, EPI_SWIGLU, T16, LO>, grid, block, 0, w, N, K, a, st, B, ep, sk, al);
+    }
   }
+  if (kind != EPI_LOGITS) return cudaErrorInvalidValue;
+  return launch_k(lc, gemv_mma_kernel<NT, EPI_LOGITS, T16, LO>, grid, block, 0, w, N, K, a, st, B, ep, sk, al);
 }
 template <int NT>
 cudaError_t gemv_nt(const LaunchCtx& lc, int kind, const void* W, int N, int K, const void* act, long long st, int B,
@@ -443,10 +445,12 @@ cudaError_t occupancy_kind(int idx) {
 }
 template <int NT>
 cudaError_t occupancy_nt(int idx) {
-  cudaError_t e = occupancy_kind<NT, EPI_QKV>(idx);
-  if (e == cudaSuccess) e = occupancy_kind<NT, EPI_RESID>(idx);
-  if (e == cudaSuccess) e = occupancy_kind<NT, EPI_SWIGLU>(idx);
-  if (e == cudaSuccess) e = occupancy_kind<NT, EPI_LOGITS>(idx);
+  cudaError_t e = occupancy_kind<NT, EPI_LOGITS>(idx);
+  if constexpr (NT <= 2) {
+    if (e == cudaSuccess) e = occupancy_kind<NT, EPI_QKV>(idx);
+    if (e == cudaSuccess) e = occupancy_kind<NT, EPI_RESID>(idx);
+    if (e == cudaSuccess) e = occupancy_kind<NT, EPI_SWIGLU>(idx);
+  }
   return e;
 }
 }  // namespace

@@ -40,8 +40,8 @@ inline int chain_attrs(const LaunchCtx& lc, cudaLaunchAttribute (&attr)[2]) {
   return n;
 }
 
-// ---- decode projections (k_gemv.cu): out[b][n] = act[b] . W[n], B <= 64
-// tokens, 16 weight rows per CTA, fused epilogue `kind`. Projections with
+// ---- decode projections (k_gemv.cu): out[b][n] = act[b] . W[n], B <= 16
+// tokens (logits: 64), 16 weight rows per CTA, fused epilogue `kind`. Projections with
 // few row tiles split K over CTAs; the partial tiles go to `part` and the
 // per-tile tickets (zeroed, re-armed by the kernel) pick the CTA that sums.
 struct SplitKWork {
@@ -201,14 +201,13 @@ struct GemmMaps {
   CUtensorMap w192;  // the same weights in boxes of 192 and 224 rows (when mid)
   CUtensorMap w224;
   CUtensorMap a_lo;  // second term of a split activation operand (used when split)
-  // the same activation operand (and second term) in boxes of 16 and of 64
-  // rows: at most 16 (64) rows (decode), the ring stages hold only those
+  // the same activation operand (and second term) of gate/up and logits in boxes of 16
+  // and of 64 rows (few): at most 16 (64) rows, the ring stages hold only those
   CUtensorMap a16;
   CUtensorMap a_lo16;
   CUtensorMap a64;
   CUtensorMap a_lo64;
-  bool has16 = false;
-  bool has64 = false;
+  bool few = false;
   bool split = false;   // the operand always has two terms (QKV, fp16 mode)
   bool has_lo = false;  // a_lo16 and a_lo64 exist
   bool mid = false;
