@@ -323,10 +323,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             tma_load_2d(sKV + s * C::TILE + c * C::CHUNK + lane * 2048, kv ? &tmV : &tmK, kv_full(s), c * 64, y);
       }
     }
-    // copies in flight land before the CTA's shared memory goes away (all
-    // were consumed unless a wait above expired)
-    if (!ok)
-      for (int i = it > NS ? it - NS : 0; i < it; ++i) mbar_wait(kv_full(i % NS), (i / NS) & 1, p.err);
+    // every copy lands before the CTA's shared memory goes away (all were consumed
+    // unless a wait ran out)
+    mbar_wait(q_full, 0, p.err);
+    for (int i = it > NS ? it - NS : 0; i < it; ++i) mbar_wait(kv_full(i % NS), (i / NS) & 1, p.err);
   } else if (warp == 9) {
     // ------------------------------------------------------------ MMA issuer
     if (lane == 0) {

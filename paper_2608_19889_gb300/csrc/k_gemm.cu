@@ -173,6 +173,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           tma_load_2d(b_at(s), &tmB, full_bar(s), kb * BK, wrow);
         }
       }
+      // every copy lands before the CTA's shared memory goes away (all were consumed
+      // unless a wait ran out)
+      for (int j = it > STAGES ? it - STAGES : 0; j < it; ++j) mbar_wait(full_bar(j % STAGES), (j / STAGES) & 1, ep.err);
     }
     __syncwarp();
   } else if (warp == 1) {
