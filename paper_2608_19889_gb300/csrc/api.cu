@@ -1850,6 +1850,13 @@ void axon_free(axon_model* m) {
   free_model(m);
 }
 
+// Not in the header: the tile width that the prefill GEMM takes for M rows and N weight
+// rows of the model's projections (tests of the width rule).
+int axon_internal_gemm_tile_n(const axon_model* m, int32_t M, int32_t N) {
+  if (!m || m->fp32 || M < 1 || N < 1) return 0;
+  return gemm_tile_n(LaunchCtx{nullptr, false, m->num_sms, m->f16}, m->m_head, M, N);
+}
+
 // Not in the header: where the flags of the persistent step's exchange stand (tests
 // of their wrap). Between steps only.
 int axon_internal_persist_epoch(axon_model* m, uint32_t epoch) {

@@ -24,9 +24,9 @@ def _built():
 @pytest.mark.parametrize("prec", ["bf16", "fp16"])
 @pytest.mark.parametrize("shape,B", [(TINY128, 12), (TINY, 16), (TINY128, 32)])
 def test_decode_batch_9_to_32(shape, B, prec):
-    """More than 8 sequences: no persistent step; the launch chain decodes
-    (GEMV projections up to 32 tokens, split-K GEMM for O and down where it
-    applies). Prefill of B x 24 rows on the tcgen05 GEMM, then 6 steps."""
+    """More than 8 sequences: no persistent step; the launch chain decodes (at
+    these widths GEMV projections of up to 16 tokens, the few-token tcgen05 kernel
+    with 32). Prefill of B x 24 rows on the tcgen05 GEMM, then 6 steps."""
     ax = _ax()
     S, n = 24, 6
     w = gpu_weights(shape)

@@ -2,6 +2,8 @@
 counts and widths at which a pass of 2,100 rows (17 row blocks on 152 SMs, the last of
 them ragged) has every projection take one of them, with whole and with cut last
 tiles. Widths of 256 and 128 are what the other prefill tests take."""
+import ctypes
+
 import pytest
 
 import synth_inputs as si
@@ -43,13 +45,16 @@ def _built():
 
 
 @pytest.mark.parametrize("prec", ["bf16", "fp16"])
-@pytest.mark.parametrize("shape", [W192, W224], ids=["192", "224"])
-def test_middle_tile_widths(shape, prec):
+@pytest.mark.parametrize("shape,width", [(W192, 192), (W224, 224)], ids=["192", "224"])
+def test_middle_tile_widths(shape, width, prec):
     ax = _ax()
     B, S = 4, 525
     w = gpu_weights(shape)
     m = create(shape, w, max_batch=B, max_context=528, fp16=prec == "fp16", max_prefill_tokens=B * S)
     try:
+        # QKV, O and down, gate/up: all take the width that the case is about
+        for n in ((shape["H"] + 2 * shape["G"]) * shape["d"], shape["D"], 2 * shape["F"]):
+            assert ax.lib().axon_internal_gemm_tile_n(m, ctypes.c_int32(B * S), ctypes.c_int32(n)) == width
         ids = si.make_ids(B, S, shape["V"], seed=7)
         lg, _ = run_prefill(m, ids, ax.AXON_LOGITS_ALL, shape["V"])
         o = oracle_for(shape, w)
