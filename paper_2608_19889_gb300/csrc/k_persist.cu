@@ -45,12 +45,15 @@
 // (last-arriver merge across splits); their cache blocks are requested before q
 // has arrived.
 //
-// Waits (persist_wait.cuh): every wait (ring mbarriers, word polls) has a limit of
-// looks, sets DEVERR_TIMEOUT and a grid-wide abort flag; after that no wait blocks, the
-// producer stops at the first ring slot whose last copy is still in flight, the kernel runs
-// to its end on garbage and the host sees the error bit. Before it exits, the producer
-// waits (bounded) for its copies in flight: the last of each slot, since none is issued
-// before the one before it has landed.
+// Waits (persist_wait.cuh): every wait has a limit of looks. A poll of words that runs
+// out sets DEVERR_TIMEOUT and a grid-wide abort flag; after that no poll blocks, the
+// weights stream to the end of the step as ever, the kernel runs to its end on garbage
+// and the host sees the error bit. (Ring waits that gave up on the abort would release
+// slots whose copies are in flight, and the producer would re-arm their barriers. To
+// look at the full barrier as well before each copy costs 2 to 3 % at 8B and 32B width.) A
+// ring wait of its own runs out only when a copy has not landed for a second or more;
+// it is reported alike, and no wait of the CTA blocks after it. Before it exits, the
+// producer waits (bounded) for its copies in flight.
 #include <type_traits>
 
 #include "attn_tile.cuh"
@@ -227,13 +230,8 @@ AXON_DEV void stream_matrix(const Ring<HD, SM>& R, const CUtensorMap* map, const
       const int slot = static_cast<int>(stage % NS);
       int ok = 1;
       if (lane == 0) {
-        // The consumers released this slot's previous use, and its copy has landed?
-        // (They release without having waited once the launch is aborting; a full
-        // barrier is not re-armed with bytes pending then either. The second look costs
-        // 8B width, 1 sequence, 2 layers 190.5 -> 193 us; 135M width 390 -> 386.)
-        if (stage >= static_cast<uint32_t>(NS))
-          ok = ring_wait(R.empty(slot), ((stage / NS) - 1) & 1u, g, s_abort, err) &&
-               mbar_try_wait(R.full(slot), ((stage / NS) - 1) & 1u);
+        if (stage >= static_cast<uint32_t>(NS))  // the consumers released this slot's previous use?
+          ok = ring_wait(R.empty(slot), ((stage / NS) - 1) & 1u, g, s_abort, err) ? 1 : 0;
         if (ok) {
           const bool two = k0 + BOXC < K;
           mbar_arrive_expect_tx(R.full(slot), two ? STAGE_BYTES : BOX_BYTES);

@@ -15,23 +15,29 @@ AXON_DEV unsigned ld_volatile(const unsigned* p) { return *reinterpret_cast<cons
 // Every wait of the step is bounded by its looks: the one that runs out sets the
 // error bit and the grid-wide abort flag, which the others see every few
 // thousand looks. (Counting looks instead of reading the clock keeps the waits
-// short: the code of a layer should fit the instruction cache.)
-AXON_DEV void wait_tick(uint32_t looks, uint32_t limit, PersistGrid* g, volatile int* s_abort, int* err) {
+// short: the code of a layer should fit the instruction cache.) s_abort, the CTA's
+// own flag: ABORT_POLLS ends its polls of words; its ring goes on as ever, since
+// copies land whatever the words hold, and no slot is released or armed out of
+// turn. ABORT_RING: a ring wait of the CTA itself ran out, and none blocks any more.
+constexpr int ABORT_POLLS = 1, ABORT_RING = 2;
+
+AXON_DEV void wait_tick(uint32_t looks, uint32_t limit, int bits, PersistGrid* g, volatile int* s_abort, int* err) {
   if ((looks & 4095u) == 0) {
     if (looks >= limit) {
       set_err(err, DEVERR_TIMEOUT);
       atomicExch(&g->abort, 1u);
+      *s_abort = bits;
     }
-    if (ld_volatile(&g->abort)) *s_abort = 1;
+    if (!*s_abort && ld_volatile(&g->abort)) *s_abort = ABORT_POLLS;
   }
 }
 
-// Wait for phase `parity` of a ring mbarrier; a no-op once the launch is aborting.
+// Wait for phase `parity` of a ring mbarrier.
 AXON_DEV bool ring_wait(uint32_t bar, uint32_t parity, PersistGrid* g, volatile int* s_abort, int* err) {
 #pragma unroll 1
   for (uint32_t looks = 0; !mbar_try_wait(bar, parity);) {
-    if (*s_abort) return false;
-    wait_tick(++looks, RING_LOOKS, g, s_abort, err);
+    if (*s_abort & ABORT_RING) return false;
+    wait_tick(++looks, RING_LOOKS, ABORT_POLLS | ABORT_RING, g, s_abort, err);
   }
   return true;
 }
@@ -66,7 +72,7 @@ AXON_DEV void poll_vecs(uint4 (&w)[N], F src, uint32_t flag, PersistGrid* g, vol
 #pragma unroll
     for (int i = 0; i < N; ++i) ok = ok && w[i].y == flag && w[i].w == flag;
     if (ok || *s_abort) return;
-    wait_tick(++looks, limit, g, s_abort, err);
+    wait_tick(++looks, limit, ABORT_POLLS, g, s_abort, err);
   }
 }
 
