@@ -734,9 +734,11 @@ struct VarlenBatch {
 // 256 364 / 364 us, 384 440 / 434, 512 480 / 467; B = 8 S = 256 1329 / 1314; 16B mixture of
 // experts, 2 layers, S = 384 459 / 450; 0.5B width, 4 layers, S = 448 270 / 278, 512 278 / 281, 640
 // 310 / 308, 1024 388 / 368, B = 16 S = 256 600 / 594; 135M width, 6 layers, S = 512 318 / 323, 640
-// 335 / 338, 768 352 / 348. Variable-length batches may hold long contexts behind short chunks (8B
-// width, 30 contexts of up to 600 tokens and a 64-token chunk: 451 / 438) and take it
-// unless they have GEMV-sized projections (at most 64 rows).
+// 335 / 338, 768 352 / 348. Variable-length batches may hold long contexts behind short
+// chunks, which the host does not know, and take it unless they have GEMV-sized projections (at most
+// 64 rows): 24 decode tokens with contexts of 64 to 300, 600 to 900 and 1500 to 2000 tokens and one or
+// two chunks of up to 100, 8B width 277 / 285, 387 / 366, 499 / 425 us; 135M width 306 / 324, 415 /
+// 387, 568 / 467.
 bool attn_on_tcgen05(int M, int S, int d, bool varlen) {
   if (varlen) return M > 64;
   return S > (d == 128 ? 384 : 576) || (S >= 256 && M >= 2048);
