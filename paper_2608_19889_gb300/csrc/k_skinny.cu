@@ -142,11 +142,7 @@ __global__ void __launch_bounds__(SK_THREADS, 2)
       for (int i = 0; i < nkb; ++i) {
         const int s = i % stages;
         ok = mbar_wait(full_bar(s), (i / stages) & 1, ep.err);
-        if (!ok) {
-          // the ring's memory is used again below: what is in flight lands first
-          for (int j = i; j < nkb && j < i + stages; ++j) mbar_wait(full_bar(j % stages), (j / stages) & 1, ep.err);
-          break;
-        }
+        if (!ok) break;
         tc_fence_after();
         const uint64_t wd = smem_desc_sw128(base + s * stage_bytes);
         const uint64_t ad = smem_desc_sw128(base + s * stage_bytes + SK_W_BYTES);
