@@ -9,6 +9,7 @@ import pytest
 import synth_inputs as si
 from helpers import LOGIT_TOL, create, gpu_weights, oracle_for
 from test_gpu_parity import _ax, check, decode_steps, oracle_decode, run_prefill
+from test_gpu_tile_widths import rounding_bound
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -80,6 +81,33 @@ def test_more_rows_than_a_token_tile(prec, oracle):
             ids = si.make_ids(B, S, WIDE["V"], seed=S)
             lg, _ = run_prefill(m, ids, ax.AXON_LOGITS_ALL, WIDE["V"])
             check(lg, o.prefill(ids, o.new_contiguous_cache(B, 160)), tol=TOL[prec], what=f"B={B} S={S} ({prec})")
+        assert ax.axon_check_device(m)[0] == 0
+    finally:
+        ax.axon_free(m)
+
+
+@pytest.mark.parametrize("prec", ["bf16", "fp16"])
+def test_qkv_too_wide_for_the_kernel(prec):
+    """41,472 weight rows of QKV are more 128-row tiles than the kernel takes: few tokens
+    run it on the GEMM's general layout, the other projections on the kernel."""
+    ax = _ax()
+    shape = dict(L=1, D=64, H=288, G=18, d=128, F=128, V=304, tie=False, bias=True, theta=1e4, eps=1e-5)
+    w = gpu_weights(shape)
+    o = oracle_for(shape, w)
+    m = create(shape, w, max_batch=9, max_context=80, fp16=prec == "fp16")
+    try:
+        for S in (9, 17, 64):
+            ids = si.make_ids(1, S, shape["V"], seed=S)
+            lg, _ = run_prefill(m, ids, ax.AXON_LOGITS_ALL, shape["V"])
+            ref = o.prefill(ids, o.new_contiguous_cache(1, 80))
+            check(lg, ref, tol=rounding_bound(ref, prec), what=f"S={S} ({prec})")
+        ids = si.make_ids(9, 5, shape["V"], seed=3)
+        _, nxt = run_prefill(m, ids, ax.AXON_LOGITS_LAST, shape["V"])
+        cache = o.new_contiguous_cache(9, 80)
+        o.prefill(ids, cache)
+        dl, fed = decode_steps(m, nxt, [5] * 9, 2, shape["V"])
+        ref = oracle_decode(o, cache, fed, [5] * 9)
+        check(dl, ref, tol=rounding_bound(ref, prec), what=f"decode of 9 ({prec})")
         assert ax.axon_check_device(m)[0] == 0
     finally:
         ax.axon_free(m)
